@@ -689,6 +689,12 @@ __global__ void __launch_bounds__(256) k_list_patch(const __grid_constant__ BoxS
 
 // MYC fluxes of the listed faces of every box (one thread per face, tiles of
 // kFaceTile consecutive entries whose first segment tile_seg gives).
+//
+// In double the kernel is bound by FP64 issue (1/64 of the FP32 rate), so
+// its time is its count of FP64 instructions: the forms of plic64.cuh took
+// it from 6.2 to 1.5 ms per sweep of the 256^3, K = 8, phi = 0.3 box (2.7 M
+// faces), and a sweep of 32^3 with 8 drops, where one warp's chain is the
+// time, from 78 to 28 us with its other launches.
 template <typename T, int NB>
 __global__ void __launch_bounds__(kFaceTile) k_face_flux_bx(const __grid_constant__ BoxSet<T, NB> S, int d,
                                                             int sweep, T band,
@@ -706,9 +712,14 @@ __global__ void __launch_bounds__(kFaceTile) k_face_flux_bx(const __grid_constan
         T st[27];
         gather_stencil_ijk(sweep_in(B, sweep) + (size_t)fc.f * B.g.N, fc.di, fc.dj, fc.dk, B.g, st);
         T m[3];
-        myc_normal(st, m);
-        const T alpha = plic_alpha_banded(m[0], m[1], m[2], st[13], band);
-        B.flux[fc.t] = face_flux(m, alpha, d, uv * B.sfac);
+        if constexpr (std::is_same<T, double>::value) {
+            myc_direction64(st, m);
+            B.flux[fc.t] = face_flux64(m, st[13], d, uv * B.sfac);
+        } else {
+            myc_normal(st, m);
+            const T alpha = plic_alpha_banded(m[0], m[1], m[2], st[13], band);
+            B.flux[fc.t] = face_flux(m, alpha, d, uv * B.sfac);
+        }
     }
 }
 

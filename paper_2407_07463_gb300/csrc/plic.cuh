@@ -2,23 +2,9 @@
 // reconstruction): the volume under a plane in the unit cube, its inverse
 // (the plane constant), Mixed-Youngs-Centred normals and split face fluxes.
 //
-// Volume.  After reflecting negative normal components (x_i -> 1 - x_i) and
-// sorting, 0 <= a <= b <= c.  With A(beta) the area of {(y,z) in [0,1]^2 :
-// b y + c z < beta} -- a piecewise quadratic with breaks at 0, b, c, b + c --
-// the volume is the mean of A over beta in [alpha - a, alpha].  Splitting
-// that interval at the breaks and integrating each quadratic piece with the
-// two-point Gauss-Legendre rule is exact, needs no division by a small
-// product (unlike the inclusion-exclusion closed form of Scardovelli &
-// Zaleski 2000, JCP 164, whose region-3 numerator cancels when a -> 0) and
-// keeps every term non-negative.
-//
-// Inverse.  The volume is convex on [0, S/2] (the cross-section area of a
-// cube grows towards its centre), so the region is located from the volumes
-// at the breaks, the closed-form roots are used in regions 1, 2 and the
-// prism region, Newton on the cubic polynomial (started from the right end of
-// the region, hence monotone) in regions 3 and 4, and one Newton step on the
-// exact piecewise form above polishes every root.  (The FP32 piecewise
-// inversion, alpha_sorted_pw below, takes regions 3 and 4 in closed form.)
+// The FP32 forms (volume, its inverse in closed form) are below; the FP64
+// forms are in plic64.cuh, which plic_volume<double>, plic_alpha<double> and
+// myc_normal(const double*) call.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -26,101 +12,14 @@
 
 #include <type_traits>
 
+#include "plic64.cuh"
+
 namespace vof {
 
-template <typename T>
-struct PlicConst;
-template <>
-struct PlicConst<double> {
-    static constexpr double half_inv_sqrt3 = 0.28867513459481288225;  // 1/(2 sqrt 3)
-    static constexpr double tiny = 1e-300;
-    static constexpr int newton_iters = 40;
-    static constexpr double newton_rtol = 4e-16;
-};
-template <>
-struct PlicConst<float> {
-    static constexpr float half_inv_sqrt3 = 0.28867513459481288225f;
-    static constexpr float tiny = 1e-30f;
-    static constexpr int newton_iters = 20;
-    static constexpr float newton_rtol = 2e-7f;
-};
+constexpr float kTinyF = 1e-30f;  // a component this small counts as zero
 
-__device__ __forceinline__ double cbrt_t(double v) { return cbrt(v); }
-__device__ __forceinline__ float cbrt_t(float v) { return cbrtf(v); }
 __device__ __forceinline__ double sqrt_t(double v) { return sqrt(v); }
 __device__ __forceinline__ float sqrt_t(float v) { return sqrtf(v); }
-
-// Area of {(y,z) in [0,1]^2 : a y + b z < beta}, 0 <= a <= b.
-template <typename T>
-__device__ __forceinline__ T area2(T a, T b, T beta) {
-    if (beta <= T(0)) return T(0);
-    T ab = a + b;
-    if (beta >= ab) return T(1);
-    if (a <= T(0)) return beta / b;
-    if (beta < a) return beta * beta / (T(2) * a * b);
-    if (beta < b) return (T(2) * beta - a) / (T(2) * b);
-    T r = ab - beta;
-    return T(1) - r * r / (T(2) * a * b);
-}
-
-// d area2 / d beta.
-template <typename T>
-__device__ __forceinline__ T area2_d(T a, T b, T beta) {
-    T ab = a + b;
-    if (beta <= T(0) || beta >= ab) return T(0);
-    if (a <= T(0)) return T(1) / b;
-    if (beta < a) return beta / (a * b);
-    if (beta < b) return T(1) / b;
-    return (ab - beta) / (a * b);
-}
-
-// Volume for sorted 0 <= a <= b <= c (c > 0), any alpha; piecewise Gauss.
-// The mean of A over [alpha - a, alpha] is taken with the widths of the
-// pieces as they are in floating point (their sum, not a, is the divisor):
-// alpha - a rounds, and dividing by a would leave an error of ulp(alpha)/a.
-template <typename T>
-__device__ __noinline__ T vol_sorted(T a, T b, T c, T alpha) {
-    T lo = alpha - a, hi = alpha;
-    if (a <= PlicConst<T>::tiny || !(hi > lo)) return area2(b, c, alpha);
-    T acc = T(0), wsum = T(0);
-    T u = lo;
-    const T br[4] = {T(0), b, c, b + c};
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-        T v = q < 4 ? br[q] : hi;
-        if (v > hi) v = hi;
-        if (v > u) {
-            T h = v - u;
-            T mid = T(0.5) * (u + v);
-            T off = h * PlicConst<T>::half_inv_sqrt3;
-            acc += h * (area2(b, c, mid - off) + area2(b, c, mid + off));
-            wsum += h;
-            u = v;
-        }
-    }
-    return T(0.5) * acc / wsum;
-}
-
-template <typename T>
-__device__ T dvol_sorted(T a, T b, T c, T alpha) {
-    T lo = alpha - a, hi = alpha;
-    if (a <= PlicConst<T>::tiny || !(hi > lo)) return area2_d(b, c, alpha);
-    T acc = T(0), wsum = T(0);
-    T u = lo;
-    const T br[4] = {T(0), b, c, b + c};
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-        T v = q < 4 ? br[q] : hi;
-        if (v > hi) v = hi;
-        if (v > u) {
-            T h = v - u;
-            acc += h * area2_d(b, c, T(0.5) * (u + v));
-            wsum += h;
-            u = v;
-        }
-    }
-    return acc / wsum;
-}
 
 template <typename T>
 __device__ __forceinline__ void sort3(T& a, T& b, T& c) {
@@ -162,11 +61,11 @@ __device__ __forceinline__ VolPW vol_pw_make(float a, float b, float c) {
     p.c = c;
     p.S = a + b + c;
     p.ab = a + b;
-    const bool b0 = b <= PlicConst<float>::tiny;
+    const bool b0 = b <= kTinyF;
     p.x_lin = b0 ? -1.f : (c >= p.ab ? p.ab : INFINITY);
     p.i6bc = 1.f / (6.f * b * c);
     const float i6abc = p.i6bc / a;
-    p.i6abc = (a > PlicConst<float>::tiny && !b0 && isfinite(i6abc)) ? i6abc : 0.f;
+    p.i6abc = (a > kTinyF && !b0 && isfinite(i6abc)) ? i6abc : 0.f;
     p.k_lin = 0.5f / c;
     return p;
 }
@@ -227,10 +126,10 @@ __device__ __forceinline__ float dvol_pw(const VolPW& p, float alpha) {
 // count diverging within a warp.
 static __device__ __noinline__ float alpha_sorted_pw(const VolPW p, float v, int* region = nullptr) {
     const float a = p.a, b = p.b, c = p.c;
-    if (a <= PlicConst<float>::tiny) {
+    if (a <= kTinyF) {
         // plane parallel to one axis: the 2D area function
         if (region) *region = 0;
-        if (b <= PlicConst<float>::tiny) return c * v;
+        if (b <= kTinyF) return c * v;
         const float t = sqrtf(2.f * b * c * v);
         return t < b ? t : c * v + 0.5f * b;
     }
@@ -282,6 +181,14 @@ __device__ __forceinline__ float alpha_pw(const VolPW& p, float cv) {
     return flip ? p.S - al : al;
 }
 
+// Power of two that brings a largest component far from one near it (1 for
+// the components that occur in a step), for the FP64 forms' products.
+__device__ __forceinline__ double scale64(double c) {
+    const int e = (int)(bits64(c) >> 52) - 1023;
+    if (e > -256 && e < 256) return 1.0;
+    return from_bits64((long long)(1023 - max(-1000, min(1000, e))) << 52);
+}
+
 // Volume of {x in [0,1]^3 : m.x < alpha}.
 template <typename T>
 __device__ __noinline__ T plic_volume(T m0, T m1, T m2, T alpha) {
@@ -294,86 +201,10 @@ __device__ __noinline__ T plic_volume(T m0, T m1, T m2, T alpha) {
     if constexpr (std::is_same<T, float>::value) {
         const float is = 1.f / S;
         return vol_pw(vol_pw_make(m0 * is, m1 * is, m2 * is), alpha * is);
-    }
-    if (alpha <= T(0)) return T(0);
-    if (alpha >= S) return T(1);
-    if (T(2) * alpha > S) return T(1) - vol_sorted(m0, m1, m2, S - alpha);
-    return vol_sorted(m0, m1, m2, alpha);
-}
-
-// Root alpha in (0, S/2] of vol_sorted(a,b,c,alpha) = v, 0 < v <= 1/2
-// (FP64; FP32 roots come from alpha_sorted_pw).  *region (if not null)
-// receives the piece the root lies in: 0 for the 2D cases (a = 0), 1..4 the
-// cubic regions, 5 the prism region.
-template <typename T>
-__device__ __noinline__ T alpha_sorted(T a, T b, T c, T v, int* region = nullptr) {
-    T al;
-    int reg;
-    if (a <= PlicConst<T>::tiny) {
-        // plane parallel to one axis: the 2D area function
-        if (region) *region = 0;
-        if (b <= PlicConst<T>::tiny) return c * v;
-        T t = sqrt_t(T(2) * b * c * v);
-        if (t < b) return t;
-        return c * v + T(0.5) * b;
-    }
-    T bc = b * c;
-    T Va = a * a / (T(6) * bc);
-    if (v <= Va) {
-        al = cbrt_t(T(6) * a * bc * v);
-        reg = 1;
     } else {
-        T Vb = (b * b - a * b + a * a / T(3)) / (T(2) * bc);
-        if (v <= Vb) {
-            T disc = T(8) * bc * v - a * a / T(3);
-            al = T(0.5) * (a + sqrt_t(disc > T(0) ? disc : T(0)));
-            reg = 2;
-        } else {
-            T ab = a + b;
-            T S = ab + c;
-            T hi;
-            bool prism = c >= ab;
-            if (prism && v >= ab / (T(2) * c)) {
-                al = c * v + T(0.5) * ab;
-                hi = T(-1);
-                reg = 5;
-            } else {
-                hi = prism ? ab : T(0.5) * S;
-                reg = 3;
-            }
-            if (hi > T(0)) {
-                // Newton on 6abc V = al^3 - (al-a)^3 - (al-b)^3 - [(al-c)^3]
-                T rhs = T(6) * a * bc * v;
-                al = hi;
-                for (int it = 0; it < PlicConst<T>::newton_iters; ++it) {
-                    T da = al - a, db = al - b, dc = al - c;
-                    T f = al * al * al - da * da * da - db * db * db - rhs;
-                    T fp = al * al - da * da - db * db;
-                    if (dc > T(0)) {
-                        f -= dc * dc * dc;
-                        fp -= dc * dc;
-                    }
-                    fp *= T(3);
-                    if (!(fp > T(0))) break;
-                    T stp = f / fp;
-                    al -= stp;
-                    if (al < b) { al = b; break; }
-                    if (fabs(stp) <= PlicConst<T>::newton_rtol * al) break;
-                }
-                if (al > c) reg = 4;
-            }
-        }
+        const double k = scale64(m2);
+        return vol64(m0 * k, m1 * k, m2 * k, alpha * k);
     }
-    // polish on the exact piecewise form
-    const T S = a + b + c;
-    const T dv = dvol_sorted(a, b, c, al);
-    const T vv = dv > T(0) ? vol_sorted(a, b, c, al) : T(0);
-    if (dv > T(0)) {
-        T nal = al - (vv - v) / dv;
-        if (nal > T(0) && nal <= T(0.5) * S) al = nal;
-    }
-    if (region) *region = reg;
-    return al;
 }
 
 // One Newton step in double on the closed form of the region the float
@@ -425,7 +256,8 @@ __device__ __noinline__ T plic_alpha(T m0, T m1, T m2, T cv) {
         const float is = 1.f / S;
         al = S * alpha_sorted_pw(vol_pw_make(m0 * is, m1 * is, m2 * is), v);
     } else {
-        al = alpha_sorted(m0, m1, m2, v);
+        const double k = scale64(m2);
+        al = alpha64_half(m0 * k, m1 * k, m2 * k, v) / k;
     }
     if (flip) al = S - al;
     return al + off;
@@ -552,6 +384,13 @@ __device__ __forceinline__ void myc_normal(const T* st, T m[3]) {
     m[0] = best[0] / n;
     m[1] = best[1] / n;
     m[2] = best[2] / n;
+}
+
+__device__ __forceinline__ void myc_normal(const double* st, double m[3]) {
+    const double il = 1.0 / myc_direction64(st, m);
+    m[0] *= il;
+    m[1] *= il;
+    m[2] *= il;
 }
 
 // Flux through a face of the donor whose reconstruction is (m, alpha); s is
