@@ -22,6 +22,7 @@ enum Slot {
     S_MISC,
     S_BITS,
     S_CCBITS,
+    S_NZ,
     S_NCMAP,
     S_MVBITS,
     S_DIL,
@@ -93,10 +94,11 @@ bool config_valid(const vof_config* c) {
 }
 
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
+size_t nz_map_bytes(size_t words) { return align256(words * sizeof(uint16_t)); }
 
 // Tiles of a face list at its largest (the list's reserved span).
 size_t list_entries_for(const vof_config* c) {
-    return (size_t)list_reserve(c->nx, c->ny, c->nz, c->k_capacity, c->precision == VOF_FP64 ? 8 : 4);
+    return (size_t)list_reserve((long long)c->ny * c->nz * ((c->nx + 31) / 32), 1, c->k_capacity);
 }
 size_t tile_cap_for(const vof_config* c) { return (list_entries_for(c) + kFaceTile - 1) / kFaceTile; }
 
@@ -117,6 +119,8 @@ Layout layout_for(const vof_config* c) {
     L.size[S_MISC] = kMiscBytes;
     L.size[S_BITS] = K * words * 4;
     L.size[S_CCBITS] = K * words * 4;
+    // maps of the words that may hold a non-zero value: of c, and of the two sweep buffers
+    L.size[S_NZ] = 3 * nz_map_bytes(words);
     L.size[S_NCMAP] = K * words * 4;
     L.size[S_MVBITS] = K * words * 4;
     // Step 4: the active fields' and the moving drops' bits dilated, plus scratch
@@ -248,14 +252,11 @@ static BoxSet<T, 1> ctx_box_set(vof_ctx* ctx, double* clipped, double dt) {
     BoxSet<T, 1> S;
     BoxDev<T>& B = S.b[0];
     const Dims& g = ctx->g;
-    const int CH = 32 * VecOf<T>::W;
     B.g = g;
     B.K = ctx->n_active;
-    B.item0 = 0;
-    B.chunk0 = 0;
-    B.cpr = (g.nx + CH - 1) / CH;
-    B.divK = fastdiv_make((uint32_t)B.K);
-    B.divcpr = fastdiv_make((uint32_t)B.cpr);
+    B.tile0 = 0;
+    B.words = g.rows * g.W;
+    B.divW = fastdiv_make((uint32_t)g.W);
     B.divny = fastdiv_make((uint32_t)g.ny);
     B.sfac = (T)(dt / ctx->cfg.h);
     B.c = (T*)ctx->c;
@@ -266,10 +267,14 @@ static BoxSet<T, 1> ctx_box_set(vof_ctx* ctx, double* clipped, double dt) {
     B.net = ctx->cfg.precision == VOF_MIXED_LEARNED ? ctx->slot<float4>(S_NET) : nullptr;
     B.ccbits = ctx->slot<uint32_t>(S_CCBITS);
     B.occbits = ctx->slot<uint32_t>(S_BITS);
+    const size_t map = nz_map_bytes((size_t)B.words) / sizeof(uint16_t);
+    B.nzc = ctx->slot<uint16_t>(S_NZ);
+    B.nz1 = B.nzc + map;
+    B.nz2 = B.nz1 + map;
     B.clipped = clipped;
     S.n = 1;
-    S.items = B.K * g.rows * B.cpr;
-    S.chunks = g.rows * B.cpr;
+    S.tw = tile_words(B.words);
+    S.tiles = (B.words + S.tw - 1) / S.tw;
     return S;
 }
 
@@ -454,7 +459,7 @@ vof_status recolour_impl(vof_ctx* ctx, int* moved_out, int* fired_out, SweepArgs
     VOF_CUDA(ctx, cudaMemcpyAsync(d_target, target.data(), (size_t)M * 4, cudaMemcpyHostToDevice, st));
     VOF_CUDA(ctx, timed(ctx, P_MOVE, [&] {
                  return recolour_move(ctx->cur, ctx->fp64, labels, ctx->slot<uint32_t>(S_MVBITS), g, mt, d_fields,
-                                     (int)hfields.size(), d_target, st);
+                                     (int)hfields.size(), d_target, ctx->slot<uint16_t>(S_NZ), st);
              }));
     ctx->launches += 1;
     if (patch && moved > 0 && ctx->n_active != na0) {
@@ -598,6 +603,8 @@ vof_status vof_init(const vof_config* cfg, void* c_dev, const void* u_dev, void*
     ctx->mlp = nullptr;
     ctx->mlp_tol = 1e-3;
     if (cudaMemsetAsync(ctx->ws + L.off[S_MISC], 0, kMiscBytes, ctx->stream) != cudaSuccess ||
+        // the sweep buffers hold anything: every word may be non-zero
+        cudaMemsetAsync(ctx->ws + L.off[S_NZ], 0xff, L.size[S_NZ], ctx->stream) != cudaSuccess ||
         cudaMemsetAsync(ctx->ws + L.off[S_HIST_R], 0, L.size[S_HIST_R], ctx->stream) != cudaSuccess ||
         cudaMemsetAsync(ctx->ws + L.off[S_HIST_RT], 0, L.size[S_HIST_RT], ctx->stream) != cudaSuccess ||
         cudaMemsetAsync(ctx->ws + L.off[S_MOM], 0, L.size[S_MOM], ctx->stream) != cudaSuccess) {
@@ -667,7 +674,6 @@ vof_status vof_step(vof_ctx* ctx, double dt, int32_t nsteps, vof_step_report* re
     a.mlp_tol = (float)ctx->mlp_tol;
     a.mlp_status = (int*)(ctx->misc() + kMiscMlpStatus);
     a.mlp_counters = mlp_counters;
-    a.update_warps = 0;
     a.update_blocks_per_sm = 0;
     int moved_total = 0, fired_steps = 0, in_use_max = -1;
     long long field_steps = 0;

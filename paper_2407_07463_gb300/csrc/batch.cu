@@ -48,18 +48,17 @@ bool batch_config_valid(const vof_batch_config* c) {
 
 // Per-box slices and shared buffers of the batch workspace.
 struct BatchLayout {
-    std::vector<size_t> b1, b2, flux, net, ccbits, occbits;
-    size_t clipped, list, counts, tile_seg, misc, vscan, total;
-    long long list_entries, items;
+    std::vector<size_t> b1, b2, flux, net, ccbits, occbits, nz;
+    size_t nz_maps, nz_bytes, clipped, list, counts, tile_seg, misc, vscan, total;
+    long long list_entries, words;
     int tile_cap;
 };
 
 BatchLayout batch_layout(const vof_batch_config* cfg, const vof_box_desc* boxes, int n) {
     BatchLayout L;
     const size_t es = cfg->precision == VOF_FP64 ? 8 : 4;
-    const int CH = (int)(512 / es);
     size_t o = 0;
-    long long items = 0, chunks = 0, kmax = 1;
+    long long words_all = 0, kmax = 1;
     for (int b = 0; b < n; ++b) {
         const vof_box_desc& d = boxes[b];
         const size_t N = (size_t)d.nx * d.ny * d.nz, K = (size_t)d.k_capacity;
@@ -70,14 +69,18 @@ BatchLayout batch_layout(const vof_batch_config* cfg, const vof_box_desc* boxes,
         L.net.push_back(o), o = al256(o + (cfg->precision == VOF_MIXED_LEARNED ? K * N * 16 : 0));
         L.ccbits.push_back(o), o = al256(o + K * words * 4);
         L.occbits.push_back(o), o = al256(o + K * words * 4);
-        items += (long long)d.k_capacity * d.ny * d.nz * ((d.nx + CH - 1) / CH);
-        chunks += (long long)d.ny * d.nz * ((d.nx + CH - 1) / CH);
+        words_all += (long long)words;
         kmax = std::max<long long>(kmax, d.k_capacity);
     }
-    L.items = items;
-    // a warp of the update pass lists up to 2 faces per cell of every field
-    // of each of its row chunks
-    L.list_entries = 2LL * CH * kmax * (chunks + 8LL * kListBlocks);
+    // maps of the words that may hold a non-zero value, three per box
+    L.nz_maps = o;
+    for (int b = 0; b < n; ++b) {
+        const size_t words = (size_t)boxes[b].ny * boxes[b].nz * ((boxes[b].nx + 31) / 32);
+        L.nz.push_back(o), o += 3 * al256(words * sizeof(uint16_t));
+    }
+    L.nz_bytes = o - L.nz_maps;
+    L.words = words_all;
+    L.list_entries = list_reserve(words_all, n, (int)kmax);
     L.tile_cap = (int)std::min<long long>((L.list_entries + kFaceTile - 1) / kFaceTile, INT32_MAX);
     L.clipped = o, o = al256(o + (size_t)n * 16 * 8);
     L.list = o, o = al256(o + 2 * (size_t)L.list_entries * 8);
@@ -102,7 +105,7 @@ struct vof_batch {
     int list_cur;
     const void* mlp;
     double mlp_tol;
-    int update_warps, update_blocks_per_sm;
+    int update_blocks_per_sm;
     float tune_ms_best;
     int tune_candidates;
     cudaGraphExec_t graphs[3][2];  // by sweep rotation and current list
@@ -116,19 +119,17 @@ namespace {
 template <typename T>
 BoxSet<T, kMaxBoxes> batch_set(vof_batch* B) {
     BoxSet<T, kMaxBoxes> S;
-    const int CH = 32 * VecOf<T>::W;
-    int item = 0, chunk = 0;
     S.n = (int)B->boxes.size();
+    S.tw = tile_words(B->L.words);
+    S.tiles = 0;
     for (int b = 0; b < S.n; ++b) {
         const vof_box_desc& d = B->boxes[b];
         BoxDev<T>& X = S.b[b];
         X.g = make_dims(d.nx, d.ny, d.nz);
         X.K = d.k_active;
-        X.item0 = item;
-        X.chunk0 = chunk;
-        X.cpr = (d.nx + CH - 1) / CH;
-        X.divK = fastdiv_make((uint32_t)X.K);
-        X.divcpr = fastdiv_make((uint32_t)X.cpr);
+        X.tile0 = S.tiles;
+        X.words = X.g.rows * X.g.W;
+        X.divW = fastdiv_make((uint32_t)X.g.W);
         X.divny = fastdiv_make((uint32_t)d.ny);
         X.sfac = (T)(d.dt / B->cfg.h);
         X.c = (T*)d.c_dev;
@@ -140,11 +141,12 @@ BoxSet<T, kMaxBoxes> batch_set(vof_batch* B) {
         X.ccbits = (uint32_t*)(B->ws + B->L.ccbits[b]);
         X.occbits = (uint32_t*)(B->ws + B->L.occbits[b]);
         X.clipped = (double*)(B->ws + B->L.clipped) + 16 * b;
-        item += X.K * X.g.rows * X.cpr;
-        chunk += X.g.rows * X.cpr;
+        const size_t map = al256((size_t)X.words * sizeof(uint16_t)) / sizeof(uint16_t);
+        X.nzc = (uint16_t*)(B->ws + B->L.nz[b]);
+        X.nz1 = X.nzc + map;
+        X.nz2 = X.nz1 + map;
+        S.tiles += (X.words + S.tw - 1) / S.tw;
     }
-    S.items = item;
-    S.chunks = chunk;
     return S;
 }
 
@@ -176,7 +178,6 @@ SweepArgs batch_args(vof_batch* B) {
     a.mlp_tol = (float)B->mlp_tol;
     a.mlp_status = (int*)(B->ws + B->L.misc);
     a.mlp_counters = (unsigned long long*)(B->ws + B->L.misc + 8);
-    a.update_warps = B->update_warps;
     a.update_blocks_per_sm = B->update_blocks_per_sm;
     return a;
 }
@@ -231,8 +232,7 @@ cudaError_t graph_step(vof_batch* B) {
 
 // Median time of `reps` first-sweep passes (listing, fluxes, update into the
 // first scratch buffer) with one launch shape; the state is not modified.
-float time_shape(vof_batch* B, int warps, int per_sm, int reps) {
-    B->update_warps = warps;
+float time_shape(vof_batch* B, int per_sm, int reps) {
     B->update_blocks_per_sm = per_sm;
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
@@ -306,11 +306,10 @@ vof_status vof_batch_init(const vof_batch_config* cfg, const vof_box_desc* boxes
     B->list_cur = 0;
     B->mlp = nullptr;
     B->mlp_tol = 1e-3;
-    // default launch shape of the update pass: 8 warps, one resident wave
-    B->update_warps = 8;
+    // default launch shape of the update pass: one resident wave
     B->update_blocks_per_sm = 1;
     {
-        const int occ = update_occupancy(fp64_batch(cfg), 8);
+        const int occ = update_occupancy(fp64_batch(cfg));
         if (occ > 0) B->update_blocks_per_sm = occ;
     }
     B->tune_ms_best = 0.f;
@@ -341,7 +340,9 @@ vof_status vof_batch_init(const vof_batch_config* cfg, const vof_box_desc* boxes
             return s;
         }
     }
-    if (cudaMemsetAsync(B->ws + B->L.clipped, 0, (size_t)n_boxes * 16 * 8, B->stream) != cudaSuccess ||
+    // the sweep buffers hold anything: every word may be non-zero
+    if (cudaMemsetAsync(B->ws + B->L.nz_maps, 0xff, B->L.nz_bytes, B->stream) != cudaSuccess ||
+        cudaMemsetAsync(B->ws + B->L.clipped, 0, (size_t)n_boxes * 16 * 8, B->stream) != cudaSuccess ||
         cudaMemsetAsync(B->ws + B->L.misc, 0, 64, B->stream) != cudaSuccess) {
         (void)cudaGetLastError();
         delete B;
@@ -369,21 +370,17 @@ vof_status vof_batch_tune(vof_batch* B) {
     if (!B) return VOF_ERR_ARG;
     if (B->sticky != VOF_OK) return B->sticky;
     if (B->cfg.precision == VOF_MIXED_LEARNED && !B->mlp) return VOF_ERR_STATE;
-    // candidates: warps per block x resident blocks per SM
+    // candidates: resident blocks per SM
     float best = INFINITY;
-    int bw = 8, bp = 0, n = 0;
-    const int warps_c[2] = {4, 8};
-    for (int w : warps_c) {
-        const int occ = update_occupancy(B->cfg.precision == VOF_FP64, w);
-        for (int p = 1; p <= std::max(1, occ); p = p < 2 ? 2 : p + 2) {
-            const float ms = time_shape(B, w, p, 3);
-            ++n;
-            if (ms < best) best = ms, bw = w, bp = p;
-        }
+    int bp = 0, n = 0;
+    const int occ = update_occupancy(B->cfg.precision == VOF_FP64);
+    for (int p = 1; p <= std::max(2, occ); p = p < 2 ? 2 : p + 2) {
+        const float ms = time_shape(B, p, 3);
+        ++n;
+        if (ms < best) best = ms, bp = p;
     }
     (void)cudaGetLastError();
     if (!std::isfinite(best)) return fail(B, VOF_ERR_CUDA);
-    B->update_warps = bw;
     B->update_blocks_per_sm = bp;
     B->tune_ms_best = best;
     B->tune_candidates = n;
@@ -458,7 +455,7 @@ vof_status vof_batch_report(vof_batch* B, vof_batch_report_t* r) {
     r->faces_network = (int64_t)cnt[0];
     r->faces_myc = (int64_t)cnt[1];
     r->faces_myc_judged = (int64_t)cnt[2];
-    r->update_warps = B->update_warps;
+    r->update_warps = kSweepThreads / 32;
     r->update_blocks_per_sm = B->update_blocks_per_sm;
     r->tune_candidates = B->tune_candidates;
     r->tune_best_ms = B->tune_ms_best;

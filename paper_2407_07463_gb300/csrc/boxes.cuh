@@ -5,13 +5,17 @@
 // The set travels by value as a __grid_constant__ kernel parameter (about
 // 8 KB for 64 boxes; read in place from the parameter space), so a
 // captured CUDA graph holds it and no table has to be copied to the
-// device.  The update and listing passes give a warp one row chunk (32 * VW
-// cells of one row of one box, VW cells per lane, 16-byte accesses) and
-// walk every field of it, so that the chunk's geometry and velocities are
-// taken once; chunks are numbered box by box, row by row, and the grid
-// walks them in bands of consecutive chunks, so that neighbouring rows and
-// planes are read close together in time (L2 reuse of c and u).  Items (one
-// field of a chunk) number the same work field by field within a chunk.
+// device.
+//
+// The sweep passes work on words: 32 consecutive cells of a row of one field
+// (the unit of the occupancy bits), VW cells per lane and 32 / VW lanes per
+// word.  Drops fill a small part of every field, so each buffer that holds a
+// state (c and the two scratch buffers) has a map of the words that may hold
+// a non-zero value (a bit per field, 16 bits per word of the grid); the
+// update pass touches only the words whose result can differ from what its
+// output buffer holds.  A tile of up to kTileWords words of one box is the
+// unit of work of a block, which lists the tile's active (word, field) items
+// in shared memory and hands them to its lane groups.
 // The face list of the next sweep holds 64-bit keys box | field | k | j | i.
 #pragma once
 
@@ -21,7 +25,6 @@
 #include "internal.h"
 #include "plic.cuh"
 #include "faces.cuh"
-#include "tc.cuh"
 #include "update_vec.cuh"
 
 namespace vof {
@@ -54,10 +57,9 @@ template <typename T>
 struct BoxDev {
     Dims g;
     int K;      // fields advected
-    int item0;  // first work item of the box
-    int chunk0; // first row chunk of the box (the update pass's unit: every field of it)
-    int cpr;    // row chunks per row, ceil(nx / (32 VW))
-    FastDiv divK, divcpr, divny;  // by K, cpr and ny
+    int tile0;  // first tile of the box
+    int words;  // 32-cell words of one field, rows * W
+    FastDiv divW, divny;  // by W and ny
     T sfac;     // dt / h
     T* c;       // [K][N] state (updated in place over a step)
     T* b1;      // [K][N] state after the first sweep
@@ -67,6 +69,9 @@ struct BoxDev {
     float4* net;        // [K][N] network normal at listed faces (learned path)
     uint32_t* ccbits;   // [K][rows][W] c > 1/2 at the step start
     uint32_t* occbits;  // [K][rows][W] c > tau after the step
+    uint16_t* nzc;      // [rows][W] fields with a non-zero value in the word of c, of b1 and of b2
+    uint16_t* nz1;      // (a set bit may stand for a word of zeros)
+    uint16_t* nz2;
     double* clipped;    // [K] volume removed by the clip
 };
 
@@ -74,8 +79,8 @@ struct BoxDev {
 template <typename T, int NB>
 struct BoxSet {
     int n;
-    int items;   // row chunk x field, over every box
-    int chunks;  // row chunks, over every box
+    int tiles;  // over every box
+    int tw;     // words per tile, at most kTileWords
     BoxDev<T> b[NB];
 };
 
@@ -85,24 +90,12 @@ __device__ __forceinline__ unsigned long long box_face_key(int box, int f, int i
 }
 
 template <typename T, int NB>
-__device__ __forceinline__ int box_of_item(const BoxSet<T, NB>& S, int it) {
+__device__ __forceinline__ int box_of_tile(const BoxSet<T, NB>& S, int tile) {
     if (NB == 1) return 0;
     int lo = 0, hi = S.n - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (S.b[mid].item0 <= it) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
-
-template <typename T, int NB>
-__device__ __forceinline__ int box_of_chunk(const BoxSet<T, NB>& S, int ch) {
-    if (NB == 1) return 0;
-    int lo = 0, hi = S.n - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (S.b[mid].chunk0 <= ch) lo = mid;
+        if (S.b[mid].tile0 <= tile) lo = mid;
         else hi = mid - 1;
     }
     return lo;
@@ -117,45 +110,61 @@ __device__ __forceinline__ T* sweep_out(const BoxDev<T>& B, int sweep) {
     return sweep == 0 ? B.b1 : (sweep == 1 ? B.b2 : B.c);
 }
 
-// Geometry of one item for lane `lane`.
-struct ItemCells {
-    int f, row, j, k, i0, x0;
-    bool valid;  // the lane's VW cells lie in the row
-    int lo_y, hi_y, lo_z, hi_z;
-};
-
-// Geometry of row chunk `chunk` of a box for lane `lane` (f = 0).
 template <typename T>
-__device__ __forceinline__ ItemCells chunk_cells(const BoxDev<T>& B, int chunk, int lane) {
-    constexpr int VW = VecOf<T>::W;
-    const Dims& g = B.g;
-    ItemCells r;
-    r.f = 0;
-    r.row = (int)fastdiv((uint32_t)chunk, B.divcpr);
-    const int seg = chunk - r.row * B.cpr;
-    const int i0 = seg * 32 * VW + lane * VW;
-    r.valid = i0 < g.nx;
-    // lanes past the row's end work on the row's first cells (every index
-    // stays in the grid) and write nothing
-    r.i0 = r.valid ? i0 : 0;
-    r.x0 = r.row * g.nx + r.i0;
-    r.k = (int)fastdiv((uint32_t)r.row, B.divny);
-    r.j = r.row - r.k * g.ny;
-    const int plane = g.nx * g.ny;
-    r.lo_y = r.j == 0 ? (g.ny - 1) * g.nx : -g.nx;
-    r.hi_y = r.j == g.ny - 1 ? -(g.ny - 1) * g.nx : g.nx;
-    r.lo_z = r.k == 0 ? (g.nz - 1) * plane : -plane;
-    r.hi_z = r.k == g.nz - 1 ? -(g.nz - 1) * plane : plane;
-    return r;
+__device__ __forceinline__ uint16_t* nz_in(const BoxDev<T>& B, int sweep) {
+    return sweep == 0 ? B.nzc : (sweep == 1 ? B.nz1 : B.nz2);
+}
+template <typename T>
+__device__ __forceinline__ uint16_t* nz_out(const BoxDev<T>& B, int sweep) {
+    return sweep == 0 ? B.nz1 : (sweep == 1 ? B.nz2 : B.nzc);
 }
 
-// Geometry of item `local` (row chunk x field) of a box for lane `lane`.
+// Words of a tile: most, and the number for a set of `words` words in all --
+// smaller tiles until they outnumber the blocks a GPU holds several times.
+constexpr int kTileWords = 128;
+constexpr int kSweepThreads = 256;
+inline int tile_words(long long words) {
+    int tw = kTileWords;
+    while (tw > 16 && words / tw < 1216) tw /= 2;
+    return tw;
+}
+
+// Place of one word of a tile.
+struct WordPlace {
+    unsigned long long key;   // face key of the word's row (field and i zero)
+    unsigned long long keyn;  // the same of the row one up along dn (dn != 0)
+    int x0, i0;               // first cell: index in the field, and along x
+    int lo, hi;               // offsets of the neighbour rows along d (d != 0)
+    int hin;                  // offset of the high neighbour row along dn (dn != 0)
+};
+
+// Place of word `word` of box `box`, with its neighbour words along d.
 template <typename T>
-__device__ __forceinline__ ItemCells item_cells(const BoxDev<T>& B, int local, int lane) {
-    const int chunk = (int)fastdiv((uint32_t)local, B.divK);
-    ItemCells r = chunk_cells(B, chunk, lane);
-    r.f = local - chunk * B.K;
-    return r;
+__device__ __forceinline__ WordPlace place_word(const BoxDev<T>& B, int box, int word, int d, int dn, int& wlo,
+                                                int& whi) {
+    const Dims& g = B.g;
+    WordPlace p;
+    const int row = (int)fastdiv((uint32_t)word, B.divW), wi = word - row * g.W;
+    const int k = (int)fastdiv((uint32_t)row, B.divny), j = row - k * g.ny;
+    p.i0 = wi * 32;
+    p.x0 = row * g.nx + p.i0;
+    // rows up and down along y and z
+    const int ylo = j == 0 ? g.ny - 1 : -1, yhi = j == g.ny - 1 ? 1 - g.ny : 1;
+    const int zlo = (k == 0 ? g.nz - 1 : -1) * g.ny, zhi = (k == g.nz - 1 ? 1 - g.nz : 1) * g.ny;
+    const int rlo = d == 1 ? ylo : zlo, rhi = d == 1 ? yhi : zhi;
+    p.lo = rlo * g.nx;
+    p.hi = rhi * g.nx;
+    wlo = d == 0 ? word + (wi == 0 ? g.W - 1 : -1) : word + rlo * g.W;
+    whi = d == 0 ? word + (wi == g.W - 1 ? 1 - g.W : 1) : word + rhi * g.W;
+    p.hin = (dn == 1 ? yhi : zhi) * g.nx;
+    p.key = box_face_key(box, 0, 0, j, k);
+    p.keyn = dn == 1 ? box_face_key(box, 0, 0, j == g.ny - 1 ? 0 : j + 1, k)
+                     : box_face_key(box, 0, 0, j, k == g.nz - 1 ? 0 : k + 1);
+    return p;
+}
+
+__device__ __forceinline__ unsigned long long key_of(unsigned long long row, int f, int i) {
+    return row | ((unsigned long long)f << 54) | (unsigned long long)i;
 }
 
 // Warp-aggregated append of nflag entries per lane to the block's segment;
@@ -173,445 +182,347 @@ __device__ __forceinline__ int warp_reserve(int nflag, int lane, int* s_count) {
     return wbase + incl - nflag;
 }
 
-// Faces of sweep d whose upwind donor is interfacial (start of a call, or
-// after a recolouring moved drops), from the state c of every box.  A warp
-// takes one row chunk and walks its fields (the velocity read once), with
-// the next field's loads issued before the current one is tested.
-template <typename T, int NB>
-__global__ void __launch_bounds__(256) k_list_bx(const __grid_constant__ BoxSet<T, NB> S, int d,
-                                                 unsigned long long* __restrict__ list, long long cap,
-                                                 int* __restrict__ counts) {
-    constexpr int VW = VecOf<T>::W;
+// Faces of sweep d whose upwind donor is interfacial, from the state c of
+// every box (start of a call, or after a field was activated), with what the
+// update pass keeps up from there on: the map of c's non-zero words and the
+// occupancy bits.  A lane group takes a word of every field in turn (the
+// velocity read once, four fields' loads in flight).
+template <typename T, int NB, int VW>
+__global__ void __launch_bounds__(kSweepThreads) k_list_sp(const __grid_constant__ BoxSet<T, NB> S, int d, T tau,
+                                                           unsigned long long* __restrict__ list, long long cap,
+                                                           int* __restrict__ counts) {
+    constexpr int LPW = 32 / VW, WPW = 32 / LPW;  // lanes per word, words per warp
+    constexpr int FB = 4;                         // fields in flight
     __shared__ int s_count;
     if (threadIdx.x == 0) s_count = 0;
     __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const int wpb = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, gl = lane & (LPW - 1);
+    const unsigned group = (0xffffffffu >> (32 - LPW)) << (lane & ~(LPW - 1));
     unsigned long long* seg = list + (size_t)blockIdx.x * cap;
-    for (int chk = blockIdx.x * wpb + (threadIdx.x >> 5); chk < S.chunks; chk += gridDim.x * wpb) {
-        const int bx = box_of_chunk(S, chk);
+    for (int tile = blockIdx.x; tile < S.tiles; tile += gridDim.x) {
+        const int bx = box_of_tile(S, tile);
         const BoxDev<T>& B = S.b[bx];
         const Dims& g = B.g;
-        const ItemCells ic = chunk_cells(B, chk - B.chunk0, lane);
-        const int x0 = ic.x0, i0 = ic.i0;
-        const int lo_d = d == 1 ? ic.lo_y : ic.lo_z;
-        const bool need_prev = lane == 0 || i0 == 0;
-        const int xp = i0 == 0 ? x0 + g.nx - 1 : x0 - 1;
-        // faces with a nonzero velocity, and those whose donor is the low cell
-        T ul[VW];
-        ld16(B.u + (size_t)d * g.N + x0, ul);
-        uint32_t nz = 0, pos = 0;
+        const int w0 = (tile - B.tile0) * S.tw, w1 = min(w0 + S.tw, B.words);
+        for (int base = w0 + (threadIdx.x >> 5) * WPW; base < w1; base += (kSweepThreads / 32) * WPW) {
+            const int word = base + lane / LPW;
+            const bool ok = word < w1;
+            int wlo, whi;
+            const WordPlace p = place_word(B, bx, ok ? word : w0, d, d, wlo, whi);
+            const bool valid = ok && p.i0 + gl * VW < g.nx;
+            const int i = p.i0 + (valid ? gl * VW : 0), x = p.x0 + (valid ? gl * VW : 0);
+            // faces of this lane's cells as donors: the low one where the
+            // velocity is negative, the high one where it is positive
+            uint32_t nlo = 0, nhi = 0;
+            {
+                T ul[VW], uh[VW];
+                const T* __restrict__ ud = B.u + (size_t)d * g.N;
+                ldv<VW>(ud + x, ul);
+                if (d == 0) {
+                    const T next = next_along_x<T, VW>(ul, ud, x, i, g.nx, gl, LPW);
 #pragma unroll
-        for (int e = 0; e < VW; ++e) {
-            const int sg = vsign(ul[e]);
-            nz |= (ic.valid && sg != 0 ? 1u : 0u) << e;
-            pos |= (sg > 0 ? 1u : 0u) << e;
-        }
-        T cx[VW], cl[VW], nx_[VW], nl[VW], pv = T(0), npv = T(0);
-        auto load = [&](int f, T (&x)[VW], T (&l)[VW], T& p) {
-            const T* cf = B.c + (size_t)f * g.N;
-            ld16(cf + x0, x);
-            if (d == 0) p = need_prev ? cf[xp] : T(0);
-            else ld16(cf + x0 + lo_d, l);
-        };
-        load(0, cx, cl, pv);
-        for (int f = 0; f < B.K; ++f) {
-            if (f + 1 < B.K) load(f + 1, nx_, nl, npv);
-            if (d == 0) {
-                T cprev = __shfl_up_sync(0xffffffffu, cx[VW - 1], 1);
-                if (need_prev) cprev = pv;
+                    for (int e = 0; e < VW; ++e) uh[e] = e == VW - 1 ? next : ul[e + 1];
+                } else {
+                    ldv<VW>(ud + x + p.hi, uh);
+                }
 #pragma unroll
-                for (int e = 0; e < VW; ++e) cl[e] = e == 0 ? cprev : cx[e - 1];
+                for (int e = 0; e < VW; ++e) {
+                    nlo |= (valid && vsign(ul[e]) < 0 ? 1u : 0u) << e;
+                    nhi |= (valid && vsign(uh[e]) > 0 ? 1u : 0u) << e;
+                }
             }
-            uint32_t fl = 0;
+            uint32_t nz = 0;
+            for (int f0 = 0; f0 < B.K; f0 += FB) {
+                T cv[FB][VW];
 #pragma unroll
-            for (int e = 0; e < VW; ++e) {
-                const T dn = (pos >> e) & 1u ? cl[e] : cx[e];
-                fl |= (((nz >> e) & 1u) && above_zero(dn) && !at_least_one(dn) ? 1u : 0u) << e;
-            }
-            if (__any_sync(0xffffffffu, fl != 0)) {
-                int p = warp_reserve(__popc(fl), lane, &s_count);
+                for (int q = 0; q < FB; ++q)
+                    if (f0 + q < B.K) ldv<VW>(B.c + (size_t)(f0 + q) * g.N + x, cv[q]);
 #pragma unroll
-                for (int e = 0; e < VW; ++e)
-                    if ((fl >> e) & 1u) seg[p++] = box_face_key(bx, f, i0 + e, ic.j, ic.k);
-            }
+                for (int q = 0; q < FB; ++q) {
+                    const int f = f0 + q;
+                    if (f >= B.K) break;
+                    bool any = false;
+                    uint32_t inter = 0, occ = 0;
 #pragma unroll
-            for (int e = 0; e < VW; ++e) {
-                cx[e] = nx_[e];
-                cl[e] = nl[e];
+                    for (int e = 0; e < VW; ++e) {
+                        any |= !is_exact_zero(cv[q][e]);
+                        inter |= (above_zero(cv[q][e]) && !at_least_one(cv[q][e]) ? 1u : 0u) << e;
+                        occ |= (above(cv[q][e], tau) ? 1u : 0u) << e;
+                    }
+                    const unsigned vote = __ballot_sync(0xffffffffu, valid && any);
+                    uint32_t ow = 0;
+                    if (vote) {  // the same for the warp
+                        if (vote & group) nz |= 1u << f;
+                        ow = gather_word<VW>(valid ? occ : 0u, lane);
+                        const uint32_t fl = inter & nlo, fh = inter & nhi;
+                        const int n = __popc(fl) + __popc(fh);
+                        if (__any_sync(0xffffffffu, n != 0)) {
+                            int pos = warp_reserve(n, lane, &s_count);
+#pragma unroll
+                            for (int e = 0; e < VW; ++e) {
+                                if ((fl >> e) & 1u) seg[pos++] = key_of(p.key, f, i + e);
+                                if ((fh >> e) & 1u)
+                                    seg[pos++] = d == 0 ? key_of(p.key, f, i + e + 1 == g.nx ? 0 : i + e + 1)
+                                                        : key_of(p.keyn, f, i + e);
+                            }
+                        }
+                    }
+                    if (ok && gl == 0) B.occbits[(size_t)f * B.words + word] = ow;
+                }
             }
-            pv = npv;
+            if (ok && gl == 0) B.nzc[word] = (uint16_t)nz;
         }
     }
     __syncthreads();
     if (threadIdx.x == 0) counts[blockIdx.x] = s_count;
 }
 
-// Stages of the update pass's copy ring: every lane keeps kUpdStages
-// (row chunk, field) items in flight through shared memory with
-// asynchronous 16-byte copies (one commit group per item), so that the
-// bytes in flight do not depend on registers.  A stage holds the item's
-// 32 * VW values of c (512 bytes per warp) and, for a y or z sweep, the same
-// chunk of its low and high neighbour rows along d; every lane reads back
-// only the 16 bytes it copied itself.
-constexpr int kUpdStages = 4;
-constexpr int kUpdRowBytes = 512;  // 32 lanes x 16 bytes
-
-__host__ __device__ constexpr int upd_rows(bool dx) { return dx ? 1 : 3; }
-__host__ __device__ constexpr size_t upd_smem_bytes(int warps, bool dx) {
-    return (size_t)warps * kUpdStages * upd_rows(dx) * kUpdRowBytes;
-}
-
-__device__ __forceinline__ void cp_async16(void* dst_smem, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(dst_smem)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-// The scalars of one field of a row chunk that do not come through the copy
-// ring: the two values beyond the chunk's ends along x that the lanes at the
-// warp's or the row's ends read (x sweep) and the c_c bit word (sweeps 1, 2).
-template <typename T>
-struct FieldScalars {
-    T pv, nv;
-    uint32_t ccw;
-};
-
-template <typename T, int PH, bool DX>
-__device__ __forceinline__ void load_field_scalars(FieldScalars<T>& r, const T* __restrict__ cf, bool need_prev,
-                                                   int xp, bool need_next, int xn,
-                                                   const uint32_t* __restrict__ ccw) {
-    if (DX) {
-        r.pv = need_prev ? cf[xp] : T(0);
-        r.nv = need_next ? cf[xn] : T(0);
-    }
-    r.ccw = PH == 0 ? 0u : *ccw;
-}
-
-// The producer side of a lane's copy ring: the next (row chunk, field) item
-// to fetch, with the chunk's source addresses computed once per chunk.
-// Lanes past a row's end copy from the row's start (in the grid; their
-// values are never used).  Every item commits one group, an empty one once
-// the warp's items are exhausted, so that waiting for all but the newest
-// kUpdStages - 1 groups always means the oldest item has landed.
-template <typename T, int NB, int PH, bool DX>
-struct UpdProducer {
-    int chk, f, K, stride, chunks;
-    const T* src;        // the lane's 16 bytes of field 0 of the chunk (sweep input)
-    size_t field_stride; // cells per field
-    int lo_d, hi_d;      // offsets of the neighbour rows along d
-
-    __device__ __forceinline__ void locate(const BoxSet<T, NB>& S, int d, int lane) {
-        if (chk >= chunks) return;
-        const BoxDev<T>& B = S.b[box_of_chunk(S, chk)];
-        const ItemCells ic = chunk_cells(B, chk - B.chunk0, lane);
-        src = sweep_in(B, PH) + ic.x0;
-        field_stride = (size_t)B.g.N;
-        K = B.K;
-        lo_d = d == 1 ? ic.lo_y : ic.lo_z;
-        hi_d = d == 1 ? ic.hi_y : ic.hi_z;
-    }
-    // Copy the next item into stage `buf` and commit its group.
-    __device__ __forceinline__ void issue(const BoxSet<T, NB>& S, int d, unsigned char* buf, int lane) {
-        if (chk < chunks) {
-            const T* row = src + (size_t)f * field_stride;
-            cp_async16(buf + lane * 16, row);
-            if (!DX) {
-                cp_async16(buf + kUpdRowBytes + lane * 16, row + lo_d);
-                cp_async16(buf + 2 * kUpdRowBytes + lane * 16, row + hi_d);
-            }
-            if (++f == K) {
-                f = 0;
-                chk += stride;
-                locate(S, d, lane);
-            }
-        }
-        cp_async_commit();
-    }
-};
-
-// Update pass of sweep PH (0, 1, 2) along d (DX: d == 0) for every box (see k_update for
-// the arithmetic): c_out = c_in - (F_hi - F_lo) + c_c (s_hi - s_lo), c_c
-// bits written in sweep 0 and read after, the clip and the occupancy bits
-// in sweep 2, and the faces of the next sweep (direction dn) whose donor is
-// interfacial appended to the block's list segment.
+// Update pass of sweep PH (0, 1, 2) along d (DX: d == 0) for every box:
+// c_out = c_in - (F_hi - F_lo) + c_c (s_hi - s_lo), c_c bits written in
+// sweep 0 and read after, the clip and the occupancy bits in sweep 2, and the
+// faces of the next sweep (direction dn) whose donor is interfacial appended
+// to the block's list segment.
 //
-// A warp takes one 32 * VW-cell row chunk at a time and walks every field
-// of it: the geometry, the velocities and their signs are taken once per
-// chunk.  The rows of c come through the copy ring: every lane keeps
-// kUpdStages (chunk, field) items in flight with asynchronous copies,
-// across the fields of a chunk and into the warp's next chunk.
-template <typename T, int NB, int PH, bool DX>
-__global__ void __launch_bounds__(256, 3) k_update_bx(const __grid_constant__ BoxSet<T, NB> S, int d, int dn,
-                                                      T tau, unsigned long long* __restrict__ nlist,
-                                                      long long cap, int* __restrict__ ncounts) {
-    constexpr int VW = VecOf<T>::W;
-    constexpr int ROWS = upd_rows(DX);
-    extern __shared__ __align__(128) unsigned char upd_smem[];
+// A word of a field is active when it, or a neighbour word along d, may be
+// non-zero in the input, or when the output buffer may hold something there
+// that has to become zero; every other word is zero in both buffers and is
+// neither read nor written (drops fill a few per cent of a field: one word in
+// five is active at phi = 0.3 in 8 fields).  The block collects the tile's
+// active (word, field) items in shared memory, so that lane groups work on
+// full items whatever their pattern; items of a word follow each other, so
+// its velocities come from L1 after the first.
+//
+// Bound: latency (three dependent loads per item: map, values, listed flux).
+// 256^3, K = 8, phi = 0.3, FP32: 0.19 ms per y or z sweep (0.38 ms when every
+// word of every field was read and written), 0.31 ms per x sweep (0.43 ms).
+template <typename T, int NB, int VW, int PH, bool DX>
+__global__ void __launch_bounds__(kSweepThreads, 4)
+    k_update_sp(const __grid_constant__ BoxSet<T, NB> S, int d, int dn, T tau,
+                unsigned long long* __restrict__ nlist, long long cap, int* __restrict__ ncounts) {
+    constexpr int LPW = 32 / VW, WPW = 32 / LPW;
+    constexpr int WARPS = kSweepThreads / 32;
     __shared__ int s_count;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int wpb = blockDim.x >> 5;
-    unsigned char* ring = upd_smem + (size_t)warp * kUpdStages * ROWS * kUpdRowBytes;
+    __shared__ int s_warp[WARPS];
+    __shared__ WordPlace s_place[kTileWords];
+    __shared__ uint16_t s_item[kTileWords * 16];  // word of the tile << 4 | field
+    __shared__ uint16_t s_cc[kTileWords];         // fields that were non-zero at the step's start
+    __shared__ uint32_t s_new[kTileWords];        // fields with a non-zero result
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, gl = lane & (LPW - 1);
+    const unsigned group = (0xffffffffu >> (32 - LPW)) << (lane & ~(LPW - 1));
     if (threadIdx.x == 0) s_count = 0;
-    __syncthreads();
-    const int sh_bits = (lane * VW) & 31;
     unsigned long long* seg = nlist + (size_t)blockIdx.x * cap;
-    const int cstride = gridDim.x * wpb;
-    // producer position (lane 0 issues; every lane tracks it) and the
-    // number of items in flight
-    UpdProducer<T, NB, PH, DX> prod;
-    prod.chk = blockIdx.x * wpb + warp;
-    prod.f = 0;
-    prod.stride = cstride;
-    prod.chunks = S.chunks;
-    prod.locate(S, d, lane);
-    auto issue_next = [&](int slot) { prod.issue(S, d, ring + (size_t)slot * ROWS * kUpdRowBytes, lane); };
-    for (int q = 0; q < kUpdStages; ++q) issue_next(q);
-    int c_slot = 0;
-    for (int chk = blockIdx.x * wpb + warp; chk < S.chunks; chk += cstride) {
-        const int bx = box_of_chunk(S, chk);
+    for (int tile = blockIdx.x; tile < S.tiles; tile += gridDim.x) {
+        const int bx = box_of_tile(S, tile);
         const BoxDev<T>& B = S.b[bx];
         const Dims& g = B.g;
-        const ItemCells ic = chunk_cells(B, chk - B.chunk0, lane);
-        const int x0 = ic.x0, i0 = ic.i0;
-        const int hi_d = d == 1 ? ic.hi_y : ic.hi_z;
-        const bool row_start = i0 == 0, row_end = i0 + VW == g.nx;
-        const bool need_prev = lane == 0 || row_start, need_next = lane == 31 || row_end;
-        const int xp = row_start ? x0 + g.nx - 1 : x0 - 1;
-        const int xn = row_end ? x0 + VW - g.nx : x0 + VW;
-        // offset from the lane's first cell to the high neighbour along d of
-        // cell e (periodic)
-        auto hi_off = [&](int e) { return DX ? (e < VW - 1 ? e + 1 : xn - x0) : e + hi_d; };
-        // velocities of the chunk: signs, s = u dt / h, and the faces of the
-        // next sweep that an interfacial cell lists
-        T s_lo[VW], s_hi[VW];
-        uint32_t lo_nz = 0, lo_pos = 0, hi_nz = 0, hi_neg = 0, nf_lo = 0, nf_hi = 0;
-        {
-            const T* __restrict__ ud = B.u + (size_t)d * g.N;
-            const T* __restrict__ udn = B.u + (size_t)dn * g.N;
-            T ulo[VW], uhi[VW], unl[VW], unh[VW];
-            ld16(ud + x0, ulo);
-            ld16(udn + x0, unl);
-            if (DX) {
-                const T unext = next_along_x<T, VW>(ulo, ud, x0, i0, g.nx, lane);
-#pragma unroll
-                for (int e = 0; e < VW; ++e) uhi[e] = e == VW - 1 ? unext : ulo[e + 1];
-            } else {
-                ld16(ud + x0 + hi_d, uhi);
-            }
-            if (dn == 0) {
-                const T nnext = next_along_x<T, VW>(unl, udn, x0, i0, g.nx, lane);
-#pragma unroll
-                for (int e = 0; e < VW; ++e) unh[e] = e == VW - 1 ? nnext : unl[e + 1];
-            } else {
-                const int hi_dn = dn == 1 ? ic.hi_y : ic.hi_z;
-                ld16(udn + x0 + hi_dn, unh);
-            }
-#pragma unroll
-            for (int e = 0; e < VW; ++e) {
-                const int sl = vsign(ulo[e]), sh = vsign(uhi[e]);
-                s_lo[e] = mul_rn(ulo[e], B.sfac);
-                s_hi[e] = mul_rn(uhi[e], B.sfac);
-                lo_nz |= (sl != 0 ? 1u : 0u) << e;
-                lo_pos |= (sl > 0 ? 1u : 0u) << e;
-                hi_nz |= (sh != 0 ? 1u : 0u) << e;
-                hi_neg |= (sh < 0 ? 1u : 0u) << e;
-                nf_lo |= (ic.valid && vsign(unl[e]) < 0 ? 1u : 0u) << e;
-                nf_hi |= (ic.valid && vsign(unh[e]) > 0 ? 1u : 0u) << e;
-            }
+        const int w0 = (tile - B.tile0) * S.tw, nw = min(S.tw, B.words - w0);
+        const int t0 = threadIdx.x;
+        uint32_t act = 0, out_old = 0;
+        if (t0 < nw) {
+            int wlo, whi;
+            s_place[t0] = place_word(B, bx, w0 + t0, d, dn, wlo, whi);
+            const uint16_t* __restrict__ in = nz_in(B, PH);
+            out_old = nz_out(B, PH)[w0 + t0];
+            act = ((uint32_t)in[w0 + t0] | in[wlo] | in[whi] | out_old) & ((1u << B.K) - 1u);
+            if (PH > 0) s_cc[t0] = PH == 2 ? (uint16_t)out_old : B.nzc[w0 + t0];
+            s_new[t0] = 0u;
         }
-        const size_t wpf = (size_t)g.rows * g.W;
-        const size_t word0 = (size_t)ic.row * g.W + (i0 >> 5);
-        const bool leader = ic.valid && (lane & (32 / VW - 1)) == 0;
-        const T* __restrict__ cin = sweep_in(B, PH);
-        T* __restrict__ cout = sweep_out(B, PH);
-        FieldScalars<T> cur, nxt;
-        load_field_scalars<T, PH, DX>(cur, cin, need_prev, xp, need_next, xn, B.ccbits + word0);
-        for (int f = 0; f < B.K; ++f) {
-            if (f + 1 < B.K)
-                load_field_scalars<T, PH, DX>(nxt, cin + (size_t)(f + 1) * g.N, need_prev, xp, need_next, xn,
-                                              B.ccbits + (size_t)(f + 1) * wpf + word0);
-            // this item's rows from the ring (the stage goes back to the
-            // producer once the item is done, every read of it consumed)
-            cp_async_wait<kUpdStages - 1>();
-            T cx[VW], cl[VW], ch[VW];
-            {
-                const unsigned char* sb = ring + (size_t)c_slot * ROWS * kUpdRowBytes + lane * 16;
-                ld16_shared(reinterpret_cast<const T*>(sb), cx);
-                if (!DX) {
-                    ld16_shared(reinterpret_cast<const T*>(sb + kUpdRowBytes), cl);
-                    ld16_shared(reinterpret_cast<const T*>(sb + 2 * kUpdRowBytes), ch);
-                }
+        // the tile's items, word by word
+        const int cnt = __popc(act);
+        int incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        if (lane == 31) s_warp[warp] = incl;
+        __syncthreads();
+        int n = 0, first = incl - cnt;
+#pragma unroll
+        for (int w = 0; w < WARPS; ++w) {
+            if (w < warp) first += s_warp[w];
+            n += s_warp[w];
+        }
+        for (uint32_t m = act; m; m &= m - 1u) s_item[first++] = (uint16_t)(t0 << 4 | (__ffs(m) - 1));
+        __syncthreads();
+        const T* __restrict__ ud = B.u + (size_t)d * g.N;
+        const T* __restrict__ udn = B.u + (size_t)dn * g.N;
+        for (int base = warp * WPW; base < n; base += WARPS * WPW) {
+            const int idx = base + lane / LPW;
+            const bool ok = idx < n;
+            const int item = s_item[ok ? idx : base];
+            const int t = item >> 4, f = item & 15;
+            const WordPlace& p = s_place[t];
+            const bool valid = ok && p.i0 + gl * VW < g.nx;
+            // lanes past a row's end work on the word's first cell and write nothing
+            const int i = p.i0 + (valid ? gl * VW : 0), x = p.x0 + (valid ? gl * VW : 0);
+            const int hi = p.hi;
+            const bool row_end = i + VW == g.nx;
+            const int xn = row_end ? x + VW - g.nx : x + VW;  // the cell after the lane's last along x
+            const T* __restrict__ cf = sweep_in(B, PH) + (size_t)f * g.N;
+            T cx[VW], cl[VW], ch[VW], ulo[VW], uhi[VW], unl[VW], unh[VW];
+            ldv<VW>(cf + x, cx);
+            ldv<VW>(ud + x, ulo);
+            ldv<VW>(udn + x, unl);
+            uint32_t ccw = 0;
+            const size_t word = (size_t)f * B.words + w0 + t;
+            if (PH > 0 && ok && ((s_cc[t] >> f) & 1u)) ccw = B.ccbits[word];
+            if (!DX) {
+                ldv<VW>(cf + x + p.lo, cl);
+                ldv<VW>(cf + x + hi, ch);
+                ldv<VW>(ud + x + hi, uhi);
             }
-            const size_t base = (size_t)f * g.N;
-            const size_t word = (size_t)f * wpf + word0;
+            if (dn != 0) ldv<VW>(udn + x + p.hin, unh);
             if (DX) {
-                T cprev = __shfl_up_sync(0xffffffffu, cx[VW - 1], 1);
-                T cnext = __shfl_down_sync(0xffffffffu, cx[0], 1);
-                if (need_prev) cprev = cur.pv;
-                if (need_next) cnext = cur.nv;
+                const bool need_prev = gl == 0, need_next = gl == LPW - 1 || row_end;
+                T cp = __shfl_up_sync(0xffffffffu, cx[VW - 1], 1), cn = __shfl_down_sync(0xffffffffu, cx[0], 1);
+                T un = __shfl_down_sync(0xffffffffu, ulo[0], 1);
+                if (need_prev) cp = cf[i == 0 ? x + g.nx - 1 : x - 1];
+                if (need_next) {
+                    cn = cf[xn];
+                    un = ud[xn];
+                }
 #pragma unroll
                 for (int e = 0; e < VW; ++e) {
-                    cl[e] = e == 0 ? cprev : cx[e - 1];
-                    ch[e] = e == VW - 1 ? cnext : cx[e + 1];
+                    cl[e] = e == 0 ? cp : cx[e - 1];
+                    ch[e] = e == VW - 1 ? cn : cx[e + 1];
+                    uhi[e] = e == VW - 1 ? un : ulo[e + 1];
                 }
+            }
+            if (dn == 0) {
+                const T un = next_along_x<T, VW>(unl, udn, x, i, g.nx, gl, LPW);
+#pragma unroll
+                for (int e = 0; e < VW; ++e) unh[e] = e == VW - 1 ? un : unl[e + 1];
             }
             uint32_t ccm = 0;
             if (PH == 0) {
-                if (ic.valid) {
+                if (valid) {
 #pragma unroll
                     for (int e = 0; e < VW; ++e) ccm |= (above_half(cx[e]) ? 1u : 0u) << e;
                 }
                 const uint32_t w = gather_word<VW>(ccm, lane);
-                if (leader) B.ccbits[word] = w;
+                if (ok && gl == 0) B.ccbits[word] = w;
             } else {
-                ccm = (cur.ccw >> sh_bits) & ((1u << VW) - 1u);
+                ccm = (ccw >> ((gl * VW) & 31)) & ((1u << VW) - 1u);
             }
-            // A warp whose cells and both neighbours along d are all empty
-            // (class 0) and carry no c_c bit has no flux through any face:
-            // every cell keeps its value and none is interfacial.
-            bool any_pos = false;
-#pragma unroll
-            for (int e = 0; e < VW; ++e) any_pos |= above_zero(cl[e]) || above_zero(cx[e]) || above_zero(ch[e]);
-            const bool quiet = !ic.valid || (ccm == 0 && !any_pos);
-            T v[VW];
-            uint32_t flo = 0, fhi = 0;
-            int nflag = 0;
-#pragma unroll
-            for (int e = 0; e < VW; ++e) v[e] = cx[e];
-            if (!__all_sync(0xffffffffu, quiet)) {
-                const T* __restrict__ flux = B.flux + base;
-#pragma unroll
-                for (int e = 0; e < VW; ++e) {
-                    // upwind donors through the low and high faces: empty (no
-                    // flux), full (flux s) or interfacial (the listed flux)
-                    const T dl = (lo_pos >> e) & 1u ? cl[e] : cx[e];
-                    const T dh = (hi_neg >> e) & 1u ? ch[e] : cx[e];
-                    const bool ml = ((lo_nz >> e) & 1u) && above_zero(dl);
-                    const bool mh = ((hi_nz >> e) & 1u) && above_zero(dh);
-                    const bool fl = at_least_one(dl), fh = at_least_one(dh);
-                    const bool cc = (ccm >> e) & 1u;
-                    T F_lo = ml && fl ? s_lo[e] : T(0), F_hi = mh && fh ? s_hi[e] : T(0);
-                    if (ml && !fl) F_lo = flux[x0 + e];
-                    if (mh && !fh) F_hi = flux[x0 + hi_off(e)];
-                    // a cell that nothing enters or leaves keeps its bits (signed zero)
-                    if (ml || mh || cc) v[e] = cx[e] - (F_hi - F_lo) + (cc ? T(1) : T(0)) * (s_hi[e] - s_lo[e]);
-                    if (PH == 2 && (v[e] < T(0) || v[e] > T(1))) continue;  // clipped below: not interfacial
-                    if (above_zero(v[e]) && !at_least_one(v[e])) {
-                        flo |= nf_lo & (1u << e);
-                        fhi |= nf_hi & (1u << e);
-                    }
-                }
-                nflag = __popc(flo) + __popc(fhi);
-            }
-            T rem[VW];
-            uint32_t occm = 0;
-            bool clipped = false;
+            T v[VW], rem[VW];
+            uint32_t flo = 0, fhi = 0, occm = 0;
+            bool nonzero = false, clipped = false;
+            const T* __restrict__ flux = B.flux + (size_t)f * g.N;
 #pragma unroll
             for (int e = 0; e < VW; ++e) {
+                // upwind donors through the low and high faces: empty (no
+                // flux), full (flux s) or interfacial (the listed flux)
+                const int sl = vsign(ulo[e]), sh = vsign(uhi[e]);
+                const T dl = sl > 0 ? cl[e] : cx[e], dh = sh < 0 ? ch[e] : cx[e];
+                const bool ml = valid && sl != 0 && above_zero(dl), mh = valid && sh != 0 && above_zero(dh);
+                const bool cc = (ccm >> e) & 1u;
+                v[e] = cx[e];
+                if (ml || mh || cc) {
+                    const T s_lo = mul_rn(ulo[e], B.sfac), s_hi = mul_rn(uhi[e], B.sfac);
+                    T F_lo = T(0), F_hi = T(0);
+                    if (ml) F_lo = at_least_one(dl) ? s_lo : flux[x + e];
+                    if (mh) F_hi = at_least_one(dh) ? s_hi : flux[DX ? (e < VW - 1 ? x + e + 1 : xn) : x + e + hi];
+                    v[e] = cx[e] - (F_hi - F_lo);
+                    if (cc) v[e] += s_hi - s_lo;
+                }
                 rem[e] = T(0);
                 if (PH == 2) {
-                    const bool clip = v[e] < T(0) || v[e] > T(1);
-                    const T cl0 = v[e] < T(0) ? T(0) : T(1);
-                    // v - cl0 is exact (Sterbenz), so the FP64 sum below sees
-                    // the same terms as a sum of FP64 differences
-                    rem[e] = clip && ic.valid ? v[e] - cl0 : T(0);
-                    clipped |= clip && ic.valid;
-                    v[e] = clip ? cl0 : v[e];
-                    if (ic.valid && v[e] > tau) occm |= 1u << e;
+                    const bool under = below_zero(v[e]), over = above(v[e], T(1));
+                    if ((under || over) && valid) {
+                        // v - 0 and v - 1 are exact (Sterbenz): the FP64 sum
+                        // below has the terms of FP64 differences
+                        const T end = under ? T(0) : T(1);
+                        rem[e] = v[e] - end;
+                        v[e] = end;
+                        clipped = true;
+                    }
+                    occm |= (valid && above(v[e], tau) ? 1u : 0u) << e;
+                }
+                nonzero |= !is_exact_zero(v[e]);
+                if (above_zero(v[e]) && !at_least_one(v[e])) {
+                    flo |= (valid && vsign(unl[e]) < 0 ? 1u : 0u) << e;
+                    fhi |= (valid && vsign(unh[e]) > 0 ? 1u : 0u) << e;
                 }
             }
-            if (ic.valid) st16(cout + base + x0, v);
+            if (valid) stv<VW>(sweep_out(B, PH) + (size_t)f * g.N + x, v);
+            const unsigned vote = __ballot_sync(0xffffffffu, valid && nonzero);
+            if (ok && gl == 0 && (vote & group)) atomicOr(&s_new[t], 1u << f);
             if (PH == 2) {
                 const uint32_t w = gather_word<VW>(occm, lane);
-                if (leader) B.occbits[word] = w;
+                if (ok && gl == 0) B.occbits[word] = w;
                 if (__any_sync(0xffffffffu, clipped)) {
                     double removed = 0.0;
 #pragma unroll
                     for (int e = 0; e < VW; ++e) removed += (double)rem[e];
-                    for (int o = 16; o > 0; o >>= 1) removed += __shfl_down_sync(0xffffffffu, removed, o);
-                    if (lane == 0 && removed != 0.0) atomicAdd(B.clipped + f, removed);
+#pragma unroll
+                    for (int o = LPW / 2; o > 0; o >>= 1) removed += __shfl_down_sync(0xffffffffu, removed, o, LPW);
+                    if (ok && gl == 0 && !is_exact_zero(removed)) atomicAdd(B.clipped + f, removed);
                 }
             }
+            const int nflag = __popc(flo) + __popc(fhi);
             if (__any_sync(0xffffffffu, nflag != 0)) {
                 int pos = warp_reserve(nflag, lane, &s_count);
 #pragma unroll
                 for (int e = 0; e < VW; ++e) {
-                    const int i = i0 + e;
-                    if ((flo >> e) & 1u) seg[pos++] = box_face_key(bx, f, i, ic.j, ic.k);
-                    if ((fhi >> e) & 1u) {
-                        int ih = i, jh = ic.j, kh2 = ic.k;
-                        if (dn == 0) ih = i + 1 == g.nx ? 0 : i + 1;
-                        else if (dn == 1) jh = ic.j + 1 == g.ny ? 0 : ic.j + 1;
-                        else kh2 = ic.k + 1 == g.nz ? 0 : ic.k + 1;
-                        seg[pos++] = box_face_key(bx, f, ih, jh, kh2);
-                    }
+                    if ((flo >> e) & 1u) seg[pos++] = key_of(p.key, f, i + e);
+                    if ((fhi >> e) & 1u)
+                        seg[pos++] = dn == 0 ? key_of(p.key, f, i + e + 1 == g.nx ? 0 : i + e + 1)
+                                             : key_of(p.keyn, f, i + e);
                 }
             }
-            cur = nxt;
-            // the item's values have been used: its stage takes the item
-            // kUpdStages ahead
-            issue_next(c_slot);
-            c_slot = c_slot + 1 == kUpdStages ? 0 : c_slot + 1;
         }
+        __syncthreads();
+        // the output's map; fields past K keep their bits
+        if (t0 < nw) {
+            const uint32_t m = s_new[t0] | (out_old & ~((1u << B.K) - 1u));
+            if (m != out_old) nz_out(B, PH)[w0 + t0] = (uint16_t)m;
+        }
+        // (the next tile's first barrier comes before anything reads what its
+        // build writes, and this thread's s_new is read above by itself)
     }
-    cp_async_wait<0>();  // nothing of this thread's is still in flight when it leaves
     __syncthreads();
     if (threadIdx.x == 0) ncounts[blockIdx.x] = s_count;
 }
 
-// Launch of the update pass of sweep `sweep` (0, 1, 2) along d.
-// Dynamic shared memory of the copy rings; the y/z instances need more than
-// the default 48 KB per block.  Every translation unit holds its own copy of
-// a kernel (no relocatable device code), so the attribute is set on the copy
-// this unit launches: internal linkage keeps one flag per unit and instance.
-template <typename T, int NB, int PH, bool DX>
-static cudaError_t update_smem_attr() {
-    static bool done = false;
-    if (done) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(k_update_bx<T, NB, PH, DX>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)upd_smem_bytes(8, DX));
-    if (e == cudaSuccess) done = true;
-    return e;
+template <typename T, int NB, int VW>
+static void launch_update_vw(const BoxSet<T, NB>& S, int d, int dn, int sweep, T tau, unsigned long long* nlist,
+                             long long cap, int* ncounts, int gb, cudaStream_t st) {
+    auto go = [&](auto kernel) { kernel<<<gb, kSweepThreads, 0, st>>>(S, d, dn, tau, nlist, cap, ncounts); };
+    if (sweep == 0) d == 0 ? go(k_update_sp<T, NB, VW, 0, true>) : go(k_update_sp<T, NB, VW, 0, false>);
+    else if (sweep == 1) d == 0 ? go(k_update_sp<T, NB, VW, 1, true>) : go(k_update_sp<T, NB, VW, 1, false>);
+    else d == 0 ? go(k_update_sp<T, NB, VW, 2, true>) : go(k_update_sp<T, NB, VW, 2, false>);
 }
 
-template <typename T, int NB, int PH>
-static cudaError_t launch_update_ph(const BoxSet<T, NB>& S, int d, int dn, T tau, unsigned long long* nlist,
-                                    long long cap, int* ncounts, int gb, int threads, cudaStream_t st) {
-    const int warps = threads / 32;
-    cudaError_t e;
-    if (d == 0) {
-        if ((e = update_smem_attr<T, NB, PH, true>()) != cudaSuccess) return e;
-        k_update_bx<T, NB, PH, true><<<gb, threads, upd_smem_bytes(warps, true), st>>>(S, d, dn, tau, nlist, cap,
-                                                                                      ncounts);
+// Launch of the update pass of sweep `sweep` (0, 1, 2) along d; vec: VecOf<T>
+// cells per lane (whole 16-byte lanes), else one.
+template <typename T, int NB>
+static cudaError_t launch_update(const BoxSet<T, NB>& S, bool vec, int d, int dn, int sweep, T tau,
+                                 unsigned long long* nlist, long long cap, int* ncounts, int gb, cudaStream_t st) {
+    if (vec) {
+        launch_update_vw<T, NB, VecOf<T>::W>(S, d, dn, sweep, tau, nlist, cap, ncounts, gb, st);
     } else {
-        if ((e = update_smem_attr<T, NB, PH, false>()) != cudaSuccess) return e;
-        k_update_bx<T, NB, PH, false><<<gb, threads, upd_smem_bytes(warps, false), st>>>(S, d, dn, tau, nlist, cap,
-                                                                                        ncounts);
+        if constexpr (NB == 1) launch_update_vw<T, NB, 1>(S, d, dn, sweep, tau, nlist, cap, ncounts, gb, st);
     }
     return cudaGetLastError();
 }
 template <typename T, int NB>
-static cudaError_t launch_update_bx(const BoxSet<T, NB>& S, int d, int dn, int sweep, T tau,
-                                    unsigned long long* nlist, long long cap, int* ncounts, int gb, int threads,
-                                    cudaStream_t st) {
-    if (sweep == 0) return launch_update_ph<T, NB, 0>(S, d, dn, tau, nlist, cap, ncounts, gb, threads, st);
-    if (sweep == 1) return launch_update_ph<T, NB, 1>(S, d, dn, tau, nlist, cap, ncounts, gb, threads, st);
-    return launch_update_ph<T, NB, 2>(S, d, dn, tau, nlist, cap, ncounts, gb, threads, st);
+static void launch_list(const BoxSet<T, NB>& S, bool vec, int d, T tau, unsigned long long* list, long long cap,
+                        int* counts, int gb, cudaStream_t st) {
+    if (vec) {
+        k_list_sp<T, NB, VecOf<T>::W><<<gb, kSweepThreads, 0, st>>>(S, d, tau, list, cap, counts);
+    } else {
+        if constexpr (NB == 1) k_list_sp<T, NB, 1><<<gb, kSweepThreads, 0, st>>>(S, d, tau, list, cap, counts);
+    }
 }
 
-// Resident blocks per SM of the y/z update pass with `warps` warps per
-// block, queried on the kernel copy of the unit that launches it.
-template <typename T, int NB>
-static int update_blocks_per_sm(int warps) {
+// Resident blocks per SM of the y/z update pass, queried on the kernel copy
+// of the unit that launches it (no relocatable device code).
+template <typename T, int NB, int VW>
+static int update_blocks_per_sm() {
     int per_sm = 0;
-    if (update_smem_attr<T, NB, 1, false>() != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_update_bx<T, NB, 1, false>, 32 * warps,
-                                                      upd_smem_bytes(warps, false)) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_update_sp<T, NB, VW, 1, false>, kSweepThreads, 0) !=
+        cudaSuccess)
         per_sm = 0;
     (void)cudaGetLastError();
     return per_sm;

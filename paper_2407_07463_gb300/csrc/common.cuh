@@ -101,6 +101,17 @@ __device__ __forceinline__ bool is_exact_zero(double v) {
 __device__ __forceinline__ bool is_exact_zero(float v) {
     return v == 0.f;
 }
+// v < 0 and v > t (t >= 0) on the bit pattern for double (false for NaN).
+__device__ __forceinline__ bool below_zero(double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    return b - 0x8000000000000001ull <= 0xFFF0000000000000ull - 0x8000000000000001ull;
+}
+__device__ __forceinline__ bool below_zero(float v) { return v < 0.f; }
+__device__ __forceinline__ bool above(double v, double t) {
+    const long long b = __double_as_longlong(v);
+    return b > (__double_as_longlong(t) & 0x7FFFFFFFFFFFFFFFLL) && b <= 0x7FF0000000000000LL;
+}
+__device__ __forceinline__ bool above(float v, float t) { return v > t; }
 // c > 1/2 (the Weymouth-Yue indicator c_c).
 __device__ __forceinline__ bool above_half(double v) {
     return __double_as_longlong(v) > 0x3FE0000000000000LL;

@@ -66,8 +66,6 @@ struct MoveTables;
 template <typename T, int NB>
 struct BoxSet;
 constexpr int kMaxBoxes = 64;
-// Largest grid of the list-producing passes.
-constexpr int kListBlocks = 2048;
 // Learned normal of a box set (FP32 path): network normals of the listed
 // faces of one sweep (tensor cores), then their judged fluxes;
 // counters[0/1] += faces on the network's / MYC's normal.
@@ -93,24 +91,19 @@ cudaError_t patch_list_fp32(const BoxSet<float, 1>& S, SweepArgs& a, int d, cons
                             const MoveTables& mt, const int* target);
 cudaError_t patch_list_fp64(const BoxSet<double, 1>& S, SweepArgs& a, int d, const uint32_t* bits, const int* labels,
                             const MoveTables& mt, const int* target);
-// Resident blocks per SM of a batch's update pass with `warps` warps per
-// block (0 if the query fails), asked of the unit that launches it.
-int update_occupancy(bool fp64, int warps);
-int update_occupancy_fp64(int warps);
+// Resident blocks per SM of a batch's update pass (0 if the query fails),
+// asked of the unit that launches it.
+int update_occupancy(bool fp64);
+int update_occupancy_fp64();
 // Listing and first sweep of a batch only (state untouched; for timing).
 cudaError_t advect_first_sweep_fp64(const BoxSet<double, kMaxBoxes>& S, SweepArgs& a);
 cudaError_t advect_first_sweep_fp32(const BoxSet<float, kMaxBoxes>& S, SweepArgs& a);
-// Face-list entries to reserve per list for K fields of grid g (either
-// sweep path, any launch shape the advance may choose): a warp of the
-// vectorised passes lists up to 2 faces per cell of every field of each of
-// its row chunks, and the segments of a grid carry the slack of their last
-// chunks.
-inline long long list_reserve(int nx, int ny, int nz, int K, int es) {
-    const long long rows = (long long)ny * nz, words = rows * ((nx + 31) / 32);
-    const long long scalar = 2LL * 32 * K * (words + kSweepBlocks);
-    const long long CH = 512 / es, cpr = (nx + CH - 1) / CH;
-    const long long vec = 2LL * CH * K * (rows * cpr + 8LL * kListBlocks);
-    return scalar > vec ? scalar : vec;
+// Face-list entries to reserve per list for up to K fields of n_boxes boxes
+// of `words` 32-cell words in all: up to 2 faces per cell of every word of
+// the blocks' tiles, a last tile per box and at least 64 blocks (sweep_grid).
+inline long long list_reserve(long long words, int n_boxes, int K) {
+    const long long padded = words + 128LL * n_boxes;
+    return 64LL * K * (padded + padded / 64 + 256);
 }
 
 // Exclusive scan of n ints (one block); off[n] = total.
@@ -205,9 +198,11 @@ cudaError_t recolour_touch(const int* labels, const uint32_t* bits, uint32_t* mv
 // The bit map of moving tags (mt.mv_map, cleared by the caller) for the
 // n_fields fields listed in mv_fields.
 cudaError_t move_map(MoveTables mt, uint32_t* map, const int* mv_fields, int n_fields, cudaStream_t st);
-// Moves the cells set in mvbits to their drop's target field.
+// Moves the cells set in mvbits to their drop's target field, whose bit of
+// the map of non-zero words (nzc, 16 bits per word) is set.
 cudaError_t recolour_move(void* c, bool fp64, const int* labels, const uint32_t* mvbits, const Dims& g,
-                          MoveTables mt, const int* mv_fields, int n_mv_fields, const int* target, cudaStream_t st);
+                          MoveTables mt, const int* mv_fields, int n_mv_fields, const int* target, uint16_t* nzc,
+                          cudaStream_t st);
 
 // Statistics helpers.
 // Per tag l <= n_max: the sum of c and its first moments about the tag's

@@ -167,13 +167,14 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_move(T* c, const int* __restrict__ labels,
                                               const uint32_t* __restrict__ mvbits, Dims g, MoveTables mt,
                                               const int* __restrict__ mv_fields, int n_mv_fields,
-                                              const int* __restrict__ target) {
+                                              const int* __restrict__ target, uint32_t* __restrict__ nzc) {
     const long long per_field = (long long)g.rows * g.W;
     const long long words = (long long)n_mv_fields * per_field;
     for (long long wd = (long long)blockIdx.x * blockDim.x + threadIdx.x; wd < words;
          wd += (long long)gridDim.x * blockDim.x) {
         uint32_t mv = mvbits[wd];
         if (!mv) continue;
+        uint32_t filled = 0;
         const int q = (int)(wd / per_field);
         const long long rem = wd - (long long)q * per_field;
         const int row = (int)(rem / g.W), wi = (int)(rem - (long long)row * g.W);
@@ -189,7 +190,9 @@ __global__ void __launch_bounds__(256) k_move(T* c, const int* __restrict__ labe
             const T v = c[(size_t)f * g.N + x];
             c[(size_t)tg * g.N + x] += v;
             c[(size_t)f * g.N + x] = T(0);
+            filled |= 1u << tg;
         }
+        if (filled) atomicOr(nzc + (rem >> 1), filled << (16 * (int)(rem & 1)));
     }
 }
 
@@ -210,14 +213,16 @@ cudaError_t move_map(MoveTables mt, uint32_t* map, const int* mv_fields, int n_f
 }
 
 cudaError_t recolour_move(void* c, bool fp64, const int* labels, const uint32_t* mvbits, const Dims& g,
-                          MoveTables mt, const int* mv_fields, int n_mv_fields, const int* target, cudaStream_t st) {
+                          MoveTables mt, const int* mv_fields, int n_mv_fields, const int* target, uint16_t* nzc,
+                          cudaStream_t st) {
     const long long words = (long long)n_mv_fields * g.rows * g.W;
+    uint32_t* nz = reinterpret_cast<uint32_t*>(nzc);
     if (fp64)
         k_move<double><<<grid_for(words, 256), 256, 0, st>>>((double*)c, labels, mvbits, g, mt, mv_fields,
-                                                            n_mv_fields, target);
+                                                            n_mv_fields, target, nz);
     else
         k_move<float><<<grid_for(words, 256), 256, 0, st>>>((float*)c, labels, mvbits, g, mt, mv_fields,
-                                                           n_mv_fields, target);
+                                                           n_mv_fields, target, nz);
     return cudaGetLastError();
 }
 
