@@ -508,25 +508,26 @@ vof_status stats_accumulate(vof_ctx* ctx, long long* D_out, double* vtot_out) {
     int* root = ctx->slot<int>(S_ROOT);
     VOF_CUDA(ctx, pack_bits(ctx->c, ctx->fp64, bits, g, ctx->n_active, occupancy_tau(ctx), st));
     ctx->launches += 1;
+    // every field tagged in one chain of launches, its drops after those of
+    // the fields before it
+    DropFields df{ctx->c, ctx->fp64, labels, bits, nout, {}, 0};
+    df.ls.n = ctx->n_active;
+    for (int f = 0; f < ctx->n_active; ++f) df.ls.f[f] = f;
+    VOF_CUDA(ctx, label_fields(bits, g, cf.connectivity, df.ls, ctx->slot<int>(S_PARENT), ctx->slot<int>(S_RANK),
+                               ctx->slot<int>(S_BTOT), ctx->slot<int>(S_BOFF), labels, nout, st, &ctx->launches, root,
+                               kDropCap));
+    int n[kMaxK];
+    VOF_CUDA(ctx, cudaMemcpyAsync(n, nout, sizeof(n), cudaMemcpyDeviceToHost, st));
+    VOF_CUDA(ctx, cudaStreamSynchronize(st));
     long long D = 0;
-    for (int f = 0; f < ctx->n_active; ++f) {
-        const char* cfp = (const char*)ctx->c + (size_t)f * g.N * ctx->es;
-        int* lab = labels + (size_t)f * g.N;
-        VOF_CUDA(ctx, label_field(bits + (size_t)f * words, g, cf.connectivity, ctx->slot<int>(S_PARENT),
-                                  ctx->slot<int>(S_RANK), ctx->slot<int>(S_BTOT), ctx->slot<int>(S_BOFF), lab,
-                                  root + D, (int)(kDropCap - D), nout + f, st, &ctx->launches));
-        int n = 0;
-        VOF_CUDA(ctx, cudaMemcpyAsync(&n, nout + f, 4, cudaMemcpyDeviceToHost, st));
-        VOF_CUDA(ctx, cudaStreamSynchronize(st));
-        if (D + n > kDropCap) return VOF_ERR_CAPACITY;
-        if (n > 0) {
-            VOF_CUDA(ctx, cudaMemsetAsync(S + 4 * D, 0, (size_t)n * 4 * 8, st));
-            VOF_CUDA(ctx, drop_sums(cfp, ctx->fp64, lab, root + D, g, S + 4 * D, n, st));
-            VOF_CUDA(ctx, drop_finalize(S + 4 * D, root + D, g, cf.h, n, vol + D, cen + 3 * D, st));
-            VOF_CUDA(ctx, drop_inertia(cfp, ctx->fp64, lab, g, cf.h, cen + 3 * D, n, shape + 6 * D, st));
-            ctx->launches += 4;
-        }
-        D += n;
+    for (int f = 0; f < ctx->n_active; ++f) D += n[f];
+    if (D > kDropCap) return VOF_ERR_CAPACITY;
+    df.n_max = (int)D;
+    if (D > 0) {
+        VOF_CUDA(ctx, drop_sums(df, g, root, S, st));
+        VOF_CUDA(ctx, drop_finalize(S, root, g, cf.h, (int)D, vol, cen, st));
+        VOF_CUDA(ctx, drop_inertia(df, g, cf.h, cen, shape, st));
+        ctx->launches += 3;
     }
     VOF_CUDA(ctx, drop_chi(shape, (int)D, shape + 6 * (size_t)kDropCap, mom + 13, st));
     std::vector<double> hvol((size_t)D);
@@ -796,20 +797,15 @@ vof_status vof_drop_table(vof_ctx* ctx, int32_t field, const int32_t* label_dev,
         (n_labels > 0 && (!vol_dev || !cen_dev)))
         return VOF_ERR_ARG;
     const Dims& g = ctx->g;
-    size_t words = (size_t)g.rows * g.W;
-    uint32_t* bits = ctx->slot<uint32_t>(S_BITS);
     const char* cf = (const char*)ctx->c + (size_t)field * g.N * ctx->es;
-    int* nout = (int*)(ctx->misc() + kMiscNout);
-    int* tmp_label = ctx->slot<int>(S_LABELS) + (size_t)field * g.N;
-    // re-derive the roots (the caller's labels must be this field's tags)
-    VOF_CUDA(ctx, pack_bits(cf, ctx->fp64, bits + (size_t)field * words, g, 1, occupancy_tau(ctx), ctx->stream));
-    VOF_CUDA(ctx, label_field(bits + (size_t)field * words, g, ctx->cfg.connectivity, ctx->slot<int>(S_PARENT),
-                              ctx->slot<int>(S_RANK), ctx->slot<int>(S_BTOT), ctx->slot<int>(S_BOFF), tmp_label,
-                              ctx->slot<int>(S_ROOT), kDropCap, nout + field, ctx->stream, &ctx->launches));
+    // a tag's root is its smallest cell, which the caller's labels hold
+    DropFields df{cf, ctx->fp64, label_dev, nullptr, nullptr, {}, n_labels};
+    df.ls.n = 1;
+    int* root = ctx->slot<int>(S_ROOT);
     double* S = ctx->slot<double>(S_DSUM);
-    VOF_CUDA(ctx, cudaMemsetAsync(S, 0, (size_t)n_labels * 4 * 8, ctx->stream));
-    VOF_CUDA(ctx, drop_sums(cf, ctx->fp64, label_dev, ctx->slot<int>(S_ROOT), g, S, n_labels, ctx->stream));
-    VOF_CUDA(ctx, drop_finalize(S, ctx->slot<int>(S_ROOT), g, ctx->cfg.h, n_labels, vol_dev, cen_dev, ctx->stream));
+    VOF_CUDA(ctx, drop_roots(df, g, root, ctx->stream));
+    VOF_CUDA(ctx, drop_sums(df, g, root, S, ctx->stream));
+    VOF_CUDA(ctx, drop_finalize(S, root, g, ctx->cfg.h, n_labels, vol_dev, cen_dev, ctx->stream));
     ctx->launches += 3;
     return VOF_OK;
 }
@@ -899,8 +895,9 @@ vof_status vof_drop_shape(vof_ctx* ctx, int32_t field, const int32_t* label_dev,
         (n_labels > 0 && (!cen_dev || !inertia_dev)))
         return VOF_ERR_ARG;
     const char* cf = (const char*)ctx->c + (size_t)field * ctx->g.N * ctx->es;
-    VOF_CUDA(ctx, drop_inertia(cf, ctx->fp64, label_dev, ctx->g, ctx->cfg.h, cen_dev, n_labels, inertia_dev,
-                               ctx->stream));
+    DropFields df{cf, ctx->fp64, label_dev, nullptr, nullptr, {}, n_labels};
+    df.ls.n = 1;
+    VOF_CUDA(ctx, drop_inertia(df, ctx->g, ctx->cfg.h, cen_dev, inertia_dev, ctx->stream));
     VOF_CUDA(ctx, drop_chi(inertia_dev, n_labels, chi_dev, nullptr, ctx->stream));
     ctx->launches += 2;
     return VOF_OK;

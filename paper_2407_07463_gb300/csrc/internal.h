@@ -137,6 +137,7 @@ cudaError_t label_field(const uint32_t* bits_f, const Dims& g, int conn, int* pa
 // sits s * N (parent, rank) and s * (nb + 1) (block totals and offsets, nb =
 // ceil(N / 1024)) from theirs.  Labels are complete only at occupied cells
 // (empty cells of a row word without an occupied cell keep what they held).
+// root_of (not null): the tags' root cells, slot after slot.
 constexpr int kLabelSlots = 16;
 struct LabelSlots {
     int n;
@@ -144,7 +145,7 @@ struct LabelSlots {
 };
 cudaError_t label_fields(const uint32_t* bits, const Dims& g, int conn, const LabelSlots& ls, int* parent, int* rank,
                          int* block_tot, int* block_off, int* labels, int* n_out, cudaStream_t st,
-                         long long* launches);
+                         long long* launches, int* root_of = nullptr, int root_cap = 0);
 // Step 3 for the slots' fields: distinct pairs of the tags of opposite
 // occupied cells around every near-contact cell, into the set `table`.
 cudaError_t tag_pairs_fields(const uint32_t* ncmap, const uint32_t* bits, const int* labels, const Dims& g, int w,
@@ -205,10 +206,25 @@ cudaError_t recolour_move(void* c, bool fp64, const int* labels, const uint32_t*
                           cudaStream_t st);
 
 // Statistics helpers.
-// Per tag l <= n_max: the sum of c and its first moments about the tag's
-// root cell root_of[l - 1] (minimum image), into S[4 (l - 1) ..].
-cudaError_t drop_sums(const void* cf, bool fp64, const int* label_f, const int* root_of, const Dims& g,
-                      double* S, int n_max, cudaStream_t st);
+// Drops of the slots' fields, counted slot after slot (a single field: one
+// slot with f[0] = 0 and its own pointers).  c and labels: the fields f * N
+// from their bases; bits (may be null): occupancy the labels were made from
+// (words without an occupied cell are skipped unread), else every label is
+// read; n_out[f]: tags of field f (null with one slot); n_max: most drops.
+struct DropFields {
+    const void* c;
+    bool fp64;
+    const int* labels;
+    const uint32_t* bits;
+    const int* n_out;
+    LabelSlots ls;
+    int n_max;
+};
+// Smallest cell of every tag (root_of[0 .. n_max)).
+cudaError_t drop_roots(const DropFields& D, const Dims& g, int* root_of, cudaStream_t st);
+// Per drop: the sum of c and its first moments about its root cell (minimum
+// image), into S[4 drop ..] (cleared first).
+cudaError_t drop_sums(const DropFields& D, const Dims& g, const int* root_of, double* S, cudaStream_t st);
 cudaError_t drop_finalize(const double* S, const int* root_of, const Dims& g, double h, int n,
                           double* vol, double* cen, cudaStream_t st);
 // Height-function curvature of one field (NaN where a cell has none) and
@@ -221,8 +237,7 @@ cudaError_t surface_tension(bool fp64, const void* c, const void* kappa, int K, 
 // first), then chi = sqrt(I_max / I_min) per drop (chi may be null) with
 // acc[0] += sum chi, acc[1] += drops, acc[2] = max(acc[2], chi) (acc may be
 // null).
-cudaError_t drop_inertia(const void* cf, bool fp64, const int* label_f, const Dims& g, double h, const double* cen,
-                         int n, double* I, cudaStream_t st);
+cudaError_t drop_inertia(const DropFields& D, const Dims& g, double h, const double* cen, double* I, cudaStream_t st);
 cudaError_t drop_chi(const double* I, int n, double* chi, double* acc, cudaStream_t st);
 cudaError_t pair_stats(const double* cen, long long n, double bx, double by, double bz, int vaxis,
                        int n_rbins, double dr, int n_tbins, double dtheta, double tie_tol, double* hist_r,
