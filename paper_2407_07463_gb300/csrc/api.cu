@@ -860,7 +860,7 @@ vof_status vof_curvature(vof_ctx* ctx, int32_t field, void* kappa_dev) {
     if (field < 0 || field >= ctx->cfg.k_capacity || !kappa_dev) return VOF_ERR_ARG;
     const char* cf = (const char*)ctx->c + (size_t)field * ctx->g.N * ctx->es;
     VOF_CUDA(ctx, timed(ctx, P_MISC, [&] {
-        return curvature_field(ctx->fp64, cf, ctx->g, ctx->cfg.h, kappa_dev, ctx->stream);
+        return curvature_fields(ctx->fp64, cf, 1, ctx->g, ctx->cfg.h, kappa_dev, true, ctx->stream);
     }));
     ctx->launches += 1;
     return VOF_OK;
@@ -874,16 +874,13 @@ vof_status vof_surface_tension(vof_ctx* ctx, double gamma, void* f_dev) {
     // the flux buffer ([K][N], the state's element type) is free between
     // calls: it holds the curvature of every active field here
     char* kap = ctx->slot<char>(S_FLUX);
-    for (int f = 0; f < ctx->n_active; ++f) {
-        const char* cf = (const char*)ctx->c + (size_t)f * g.N * ctx->es;
-        VOF_CUDA(ctx, timed(ctx, P_MISC, [&] {
-            return curvature_field(ctx->fp64, cf, g, ctx->cfg.h, kap + (size_t)f * g.N * ctx->es, ctx->stream);
-        }));
-    }
+    VOF_CUDA(ctx, timed(ctx, P_MISC, [&] {
+        return curvature_fields(ctx->fp64, ctx->c, ctx->n_active, g, ctx->cfg.h, kap, false, ctx->stream);
+    }));
     VOF_CUDA(ctx, timed(ctx, P_MISC, [&] {
         return surface_tension(ctx->fp64, ctx->c, kap, ctx->n_active, g, ctx->cfg.h, gamma, f_dev, ctx->stream);
     }));
-    ctx->launches += ctx->n_active + 1;
+    ctx->launches += 2;
     return VOF_OK;
 }
 

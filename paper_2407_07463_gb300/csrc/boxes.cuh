@@ -167,21 +167,6 @@ __device__ __forceinline__ unsigned long long key_of(unsigned long long row, int
     return row | ((unsigned long long)f << 54) | (unsigned long long)i;
 }
 
-// Warp-aggregated append of nflag entries per lane to the block's segment;
-// returns the lane's first slot.
-__device__ __forceinline__ int warp_reserve(int nflag, int lane, int* s_count) {
-    int incl = nflag;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-    }
-    int wbase = 0;
-    if (lane == 31 && incl > 0) wbase = atomicAdd(s_count, incl);
-    wbase = __shfl_sync(0xffffffffu, wbase, 31);
-    return wbase + incl - nflag;
-}
-
 // Faces of sweep d whose upwind donor is interfacial, from the state c of
 // every box (start of a call, or after a field was activated), with what the
 // update pass keeps up from there on: the map of c's non-zero words and the

@@ -143,6 +143,21 @@ __device__ __forceinline__ long long warp_append(bool flag, unsigned long long* 
     return (long long)(base + __popc(mask & ((1u << lane) - 1u)));
 }
 
+// Warp-aggregated append of nflag entries per lane to the block's segment;
+// returns the lane's first slot.
+__device__ __forceinline__ int warp_reserve(int nflag, int lane, int* s_count) {
+    int incl = nflag;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    int wbase = 0;
+    if (lane == 31 && incl > 0) wbase = atomicAdd(s_count, incl);
+    wbase = __shfl_sync(0xffffffffu, wbase, 31);
+    return wbase + incl - nflag;
+}
+
 // Bits of cells x0 .. x0+31 (periodic in nx) of one occupancy row.
 __device__ __forceinline__ uint32_t row_window(const uint32_t* __restrict__ row, int W, int nx, int x0) {
     x0 %= nx;

@@ -227,10 +227,12 @@ cudaError_t drop_roots(const DropFields& D, const Dims& g, int* root_of, cudaStr
 cudaError_t drop_sums(const DropFields& D, const Dims& g, const int* root_of, double* S, cudaStream_t st);
 cudaError_t drop_finalize(const double* S, const int* root_of, const Dims& g, double h, int n,
                           double* vol, double* cen, cudaStream_t st);
-// Height-function curvature of one field (NaN where a cell has none) and
-// the surface-tension source f[3][N] = sum over K fields of gamma kappa grad c
-// on the low faces (Section 2.3).
-cudaError_t curvature_field(bool fp64, const void* cf, const Dims& g, double h, void* kappa, cudaStream_t st);
+// Height-function curvatures of K fields (NaN where an interfacial cell has
+// none; with fill also in every other cell, which is otherwise not written)
+// and the surface-tension source f[3][N] = sum over K fields of gamma kappa
+// grad c on the low faces (Section 2.3), from curvatures of either kind.
+cudaError_t curvature_fields(bool fp64, const void* c, int K, const Dims& g, double h, void* kappa, bool fill,
+                             cudaStream_t st);
 cudaError_t surface_tension(bool fp64, const void* c, const void* kappa, int K, const Dims& g, double h,
                             double gamma, void* f, cudaStream_t st);
 // Drop shape (Appendix A): I[n][6] = xx yy zz xy xz yz about cen (cleared
