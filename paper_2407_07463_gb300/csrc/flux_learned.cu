@@ -50,23 +50,39 @@ __global__ void __launch_bounds__(128, 4) k_face_normals_net(const __grid_consta
     uint32_t phase = 0;
     const int t = threadIdx.x;
     const int n = off[nseg];
-    // the loop bound is the same for every thread of the CTA
-    for (int base = blockIdx.x * 128; base < n; base += gridDim.x * 128) {
+    const int stride = gridDim.x * 128;
+    // The stencils of the next tile are gathered while this tile's layers run
+    // (27 registers), the key of the one after that while they are: the three
+    // dependent loads of a face (key, velocity, stencil) leave the critical
+    // path.  256^3, K = 8: 0.29 ms per sweep against 0.31 gathering first.
+    auto load_key = [&](int base) -> unsigned long long {
         const int e = base + t;
-        const bool valid = e < n;
-        float st[27];
-        float4* dst = nullptr;
-        if (valid) {
-            const int sgi = segment_from(off, tile_seg[base / kFaceTile], e);
+        if (e >= n) return 0ull;
+        const int sgi = segment_from(off, tile_seg[base / kFaceTile], e);
+        return list[(size_t)sgi * cap + (e - off[sgi])];
+    };
+    float st[27];
+    float4* dst = nullptr;
+    auto gather = [&](int base, unsigned long long key) {
+        if (base + t < n) {
             float uv;
-            const BoxFace fc = decode_box_face(S, list[(size_t)sgi * cap + (e - off[sgi])], d, uv);
+            const BoxFace fc = decode_box_face(S, key, d, uv);
             const BoxDev<float>& B = S.b[fc.box];
             dst = B.net + fc.t;
             gather_stencil_ijk(sweep_in(B, sweep) + (size_t)fc.f * B.g.N, fc.di, fc.dj, fc.dk, B.g, st);
         } else {
+            dst = nullptr;
 #pragma unroll
             for (int q = 0; q < 27; ++q) st[q] = 0.5f;
         }
+    };
+    unsigned long long key = 0ull;
+    if ((int)blockIdx.x * 128 < n) {
+        gather(blockIdx.x * 128, load_key(blockIdx.x * 128));
+        key = load_key(blockIdx.x * 128 + stride);
+    }
+    // the loop bound is the same for every thread of the CTA
+    for (int base = blockIdx.x * 128; base < n; base += stride) {
         CanonFrame fr;
         canon_frame(st, fr);
         // the stencil through this thread's scratch column, so that the
@@ -77,12 +93,17 @@ __global__ void __launch_bounds__(128, 4) k_face_normals_net(const __grid_consta
         float x[27];
         canon_input_col(col, 128, fr, x);
         store_input_row(s, t, x);
+        float4* const out = dst;
         float oc[3];
-        if (!mlp_tile_forward(s, taddr, phase, oc)) break;
-        if (valid) {
+        const bool alive = mlp_tile_forward(s, taddr, phase, oc, [&] {
+            gather(base + stride, key);
+            key = load_key(base + 2 * stride);
+        });
+        if (!alive) break;
+        if (out) {
             float nn[3];
             canon_output(oc, fr, nn);
-            *dst = make_float4(nn[0], nn[1], nn[2], 0.f);
+            *out = make_float4(nn[0], nn[1], nn[2], 0.f);
         }
     }
     mlp_cta_end(s, status);

@@ -111,8 +111,9 @@ __device__ __forceinline__ void store_pairs8(unsigned char* tile, int r, int k0,
     for (int q = 0; q < 4; ++q) {
         // split_bf16 on two values at once: one packed conversion per part
         const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
-        const float2 hf = __bfloat1622float2(h);
-        const __nv_bfloat162 l = __floats2bfloat162_rn(v[2 * q] - hf.x, v[2 * q + 1] - hf.y);
+        // v - hi for both in one packed operation (exact product by -1)
+        const float2 r = __ffma2_rn(__bfloat1622float2(h), make_float2(-1.f, -1.f), make_float2(v[2 * q], v[2 * q + 1]));
+        const __nv_bfloat162 l = __floats2bfloat162_rn(r.x, r.y);
         hi[q] = *reinterpret_cast<const uint32_t*>(&h);
         lo[q] = *reinterpret_cast<const uint32_t*>(&l);
     }

@@ -25,7 +25,8 @@ struct MlpSmem {
     unsigned char W1[kHid * kIn * 2];    // 64 x 32
     unsigned char W2[kHid * kHid * 2];   // 64 x 64
     unsigned char W3[kOutP * kHid * 2];  // 16 x 64
-    float b1[kHid], b2[kHid], b3[kOutP];
+    alignas(16) float b1[kHid];
+    float b2[kHid], b3[kOutP];
     uint64_t bar;
     uint32_t tbase;
     int timeout;
@@ -97,9 +98,23 @@ __device__ __forceinline__ bool finish_layer(MlpSmem& s, uint32_t& phase) {
     return true;
 }
 
+// v = max(v + b, 0) for 32 values, the sums two at a time.
+__device__ __forceinline__ void bias_relu(float v[32], const float* b) {
+    const float2* b2 = reinterpret_cast<const float2*>(b);
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+        const float2 r = __fadd2_rn(make_float2(v[2 * q], v[2 * q + 1]), b2[q]);
+        v[2 * q] = fmaxf(r.x, 0.f);
+        v[2 * q + 1] = fmaxf(r.y, 0.f);
+    }
+}
+
 // Forward pass of the tile whose canonical inputs are in s.H.  out[3] gets
 // this thread's canonical output.  Every thread of the CTA must call it.
-__device__ __forceinline__ bool mlp_tile_forward(MlpSmem& s, uint32_t taddr, uint32_t& phase, float out[3]) {
+// overlap() runs while the first layer is on the tensor cores.
+template <typename F>
+__device__ __forceinline__ bool mlp_tile_forward(MlpSmem& s, uint32_t taddr, uint32_t& phase, float out[3],
+                                                 F&& overlap) {
     const int t = threadIdx.x;
     const uint32_t lane_off = (uint32_t)(32 * (t >> 5)) << 16;
     tc::fence_async_smem();
@@ -107,12 +122,12 @@ __device__ __forceinline__ bool mlp_tile_forward(MlpSmem& s, uint32_t taddr, uin
     __syncthreads();
     tc::fence_after_sync();
     if (t == 0) issue_layer(taddr + kColD1, s.H, kInHL, s.W1, kIn, kHid, &s.bar);
+    overlap();
     if (!finish_layer(s, phase)) return false;
     for (int c0 = 0; c0 < kHid; c0 += 32) {
         float v[32];
         tc::tmem_ld32(taddr + lane_off + kColD1 + c0, v);
-#pragma unroll
-        for (int q = 0; q < 32; ++q) v[q] = fmaxf(v[q] + s.b1[c0 + q], 0.f);
+        bias_relu(v, s.b1 + c0);
 #pragma unroll
         for (int k8 = 0; k8 < 32; k8 += 8) store_pairs8(s.H, t, c0 + k8, kHid, kHidHL, v + k8);
     }
@@ -126,8 +141,7 @@ __device__ __forceinline__ bool mlp_tile_forward(MlpSmem& s, uint32_t taddr, uin
     for (int c0 = 0; c0 < kHid; c0 += 32) {
         float v[32];
         tc::tmem_ld32(taddr + lane_off + kColD2 + c0, v);
-#pragma unroll
-        for (int q = 0; q < 32; ++q) v[q] = fmaxf(v[q] + s.b2[c0 + q], 0.f);
+        bias_relu(v, s.b2 + c0);
 #pragma unroll
         for (int k8 = 0; k8 < 32; k8 += 8) store_pairs8(s.H, t, c0 + k8, kHid, kHidHL, v + k8);
     }
@@ -143,6 +157,10 @@ __device__ __forceinline__ bool mlp_tile_forward(MlpSmem& s, uint32_t taddr, uin
     out[1] = v[1] + s.b3[1];
     out[2] = v[2] + s.b3[2];
     return true;
+}
+
+__device__ __forceinline__ bool mlp_tile_forward(MlpSmem& s, uint32_t taddr, uint32_t& phase, float out[3]) {
+    return mlp_tile_forward(s, taddr, phase, out, [] {});
 }
 
 __device__ __forceinline__ void mlp_cta_begin(MlpSmem& s, const MlpBlob* w) {
