@@ -33,12 +33,9 @@ namespace vof {
 
 // Buffers and settings shared by the boxes of one advance (internal).
 struct SweepArgs {
-    unsigned long long* list;    // two face lists of list_entries entries each, segmented by block
+    unsigned long long* list;    // two face lists of list_entries entries each
     long long list_entries;      // reserved entries per list
-    int* counts;                 // [2][kSweepBlocks] segment lengths
-    int* offsets;                // [kSweepBlocks + 1] scan of the current counts
-    int* tile_seg;               // first segment of each tile of kFaceTile listed faces
-    int tile_cap;
+    int* counts;                 // [2] their lengths
     long long step;              // index of the first step
     double band;                 // FP64 plane-constant band (FP32 path)
     double tau;                  // occupancy threshold
@@ -56,10 +53,6 @@ struct SweepArgs {
 };
 
 
-// Face lists are segmented by block: block b of the listing kernels owns
-// list[b * cap .. b * cap + count[b]), filled through a shared-memory counter,
-// so no global atomic is contended.
-
 // Rows of whole 16-byte lanes on 16-byte-aligned buffers take VW cells per
 // lane, others (a context only) one.
 template <typename T, int NB>
@@ -69,48 +62,42 @@ inline bool rows_vectorisable(const BoxSet<T, NB>& S) {
     return B.g.nx % VecOf<T>::W == 0 && (((uintptr_t)B.c | (uintptr_t)B.u) & 15) == 0;
 }
 
-// Grid and per-block list capacity of one advance; every producer of a list
-// in it uses the same grid so that the consumers' segment walk is uniform.
-struct SweepGrid {
-    int gb;
-    long long cap;
-};
-
-// Every block takes the same number of tiles (up to the last block's rest):
-// the fewest that the resident blocks can share out.
+// Blocks of a list-writing pass: every block takes the same number of tiles
+// (up to the last block's rest), the fewest that the resident blocks can
+// share out.
 template <typename T, int NB>
-SweepGrid sweep_grid(const BoxSet<T, NB>& S, bool vec, const SweepArgs& a) {
-    SweepGrid r;
+int sweep_grid(const BoxSet<T, NB>& S, bool vec, const SweepArgs& a) {
     int per_sm = a.update_blocks_per_sm;
     if (per_sm <= 0) per_sm = std::max(1, vec ? update_blocks_per_sm<T, NB, VecOf<T>::W>() : update_blocks_per_sm<T, NB, 1>());
-    const int most = std::max(64, std::min(kSweepBlocks, sm_count() * per_sm));
+    const int most = sm_count() * per_sm;
     const int per_block = (S.tiles + most - 1) / most;
-    r.gb = (S.tiles + per_block - 1) / per_block;
-    int kmax = 1;
-    for (int b = 0; b < S.n; ++b) kmax = std::max(kmax, S.b[b].K);
-    r.cap = 64LL * kmax * S.tw * per_block;  // up to 2 faces per cell and field
-    return r;
+    return (S.tiles + per_block - 1) / per_block;
+}
+
+// Whether the reserved lists hold every face the set can list.
+template <typename T, int NB>
+bool lists_fit(const BoxSet<T, NB>& S, const SweepArgs& a) {
+    long long need = 0;
+    for (int b = 0; b < S.n; ++b) need += list_reserve(S.b[b].words, S.b[b].K);
+    return need <= a.list_entries;
 }
 
 template <typename T, int NB>
-void face_fluxes(const BoxSet<T, NB>& S, int d, int sweep, const unsigned long long* list, long long cap, int gb,
-                 SweepArgs& a) {
+void face_fluxes(const BoxSet<T, NB>& S, int d, int sweep, const unsigned long long* list, const int* count,
+                 int* next_count, SweepArgs& a) {
     if constexpr (std::is_same<T, float>::value) {
         if (a.mlp) {
             if (a.prof) a.prof->begin(P_NET_NORMALS);
-            face_normals_net_set<NB>(S, d, sweep, list, cap, a.offsets, gb, a.tile_seg, a.mlp, a.mlp_status,
-                                     a.stream);
+            face_normals_net_set<NB>(S, d, sweep, list, count, next_count, a.mlp, a.mlp_status, a.stream);
             if (a.prof) { a.prof->end(); a.prof->begin(P_FACE_FLUX); }
-            face_flux_judged_set<NB>(S, d, sweep, (float)a.band, list, cap, a.offsets, gb, a.tile_seg, a.mlp_tol,
-                                     a.mlp_counters, a.stream);
+            face_flux_judged_set<NB>(S, d, sweep, (float)a.band, list, count, a.mlp_tol, a.mlp_counters, a.stream);
             if (a.prof) a.prof->end();
             if (a.launches) *a.launches += 2;
             return;
         }
     }
     if (a.prof) a.prof->begin(P_FACE_FLUX);
-    k_face_flux_bx<T, NB><<<sm_count() * 16, kFaceTile, 0, a.stream>>>(S, d, sweep, (T)a.band, list, cap, a.offsets, gb,
-                                                                 a.tile_seg);
+    k_face_flux_bx<T, NB><<<sm_count() * 16, kFaceTile, 0, a.stream>>>(S, d, sweep, (T)a.band, list, count, next_count);
     if (a.prof) a.prof->end();
     if (a.launches) *a.launches += 1;
 }
@@ -121,17 +108,19 @@ template <typename T, int NB>
 cudaError_t advect_set(const BoxSet<T, NB>& S, SweepArgs& a, int nsteps) {
     if (S.n == 0 || nsteps <= 0) return cudaSuccess;
     const bool vec = rows_vectorisable(S);
-    const SweepGrid G = sweep_grid(S, vec, a);
-    if ((long long)G.gb * G.cap > a.list_entries || G.gb > kSweepBlocks) return cudaErrorInvalidValue;
+    const int gb = sweep_grid(S, vec, a);
+    if (!lists_fit(S, a)) return cudaErrorInvalidValue;
     unsigned long long* lists[2] = {a.list, a.list + a.list_entries};
-    int* counts[2] = {a.counts, a.counts + kSweepBlocks};
+    int* counts[2] = {a.counts, a.counts + 1};
     const T tau = (T)a.tau;
     for (int s = 0; s < nsteps; ++s) {
         const long long step = a.step + s;
         const int rot = (int)(step % 3);
         if (!a.list_valid) {
             if (a.prof) a.prof->begin(P_FIND_FACES);
-            launch_list(S, vec, rot, tau, lists[a.list_cur], G.cap, counts[a.list_cur], G.gb, a.stream);
+            const cudaError_t z = cudaMemsetAsync(counts[a.list_cur], 0, sizeof(int), a.stream);
+            if (z != cudaSuccess) return z;
+            launch_list(S, vec, rot, tau, lists[a.list_cur], counts[a.list_cur], gb, a.stream);
             if (a.prof) a.prof->end();
             if (a.launches) *a.launches += 1;
             cudaError_t e = cudaGetLastError();
@@ -144,15 +133,11 @@ cudaError_t advect_set(const BoxSet<T, NB>& S, SweepArgs& a, int nsteps) {
             const int cur = a.list_cur, nxt = 1 - a.list_cur;
             // every launch's error is taken where it happens (a later launch's
             // query would clear it)
-            if (a.prof) a.prof->begin(P_SCAN);
-            cudaError_t e = scan_face_counts(counts[cur], a.offsets, G.gb, a.tile_seg, a.tile_cap, a.stream);
-            if (a.launches) *a.launches += 1;
-            if (a.prof) a.prof->end();
+            face_fluxes(S, d, sw, lists[cur], counts[cur], counts[nxt], a);
+            cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) return e;
-            face_fluxes(S, d, sw, lists[cur], G.cap, G.gb, a);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
             if (a.prof) a.prof->begin(P_UPDATE);
-            e = launch_update(S, vec, d, dn, sw, tau, lists[nxt], G.cap, counts[nxt], G.gb, a.stream);
+            e = launch_update(S, vec, d, dn, sw, tau, lists[nxt], counts[nxt], gb, a.stream);
             if (e != cudaSuccess) {
                 if (a.prof) a.prof->end();
                 return e;
@@ -173,12 +158,8 @@ template <typename T>
 cudaError_t patch_list_set(const BoxSet<T, 1>& S, SweepArgs& a, int d, const uint32_t* bits, const int* labels,
                            const MoveTables& mt, const int* target) {
     if (!a.list_valid) return cudaSuccess;
-    const bool vec = rows_vectorisable(S);
-    const SweepGrid G = sweep_grid(S, vec, a);
     unsigned long long* list = a.list + (a.list_cur ? a.list_entries : 0);
-    const int* counts = a.counts + (a.list_cur ? kSweepBlocks : 0);
-    k_list_patch<T><<<std::min(G.gb, sm_count() * 8), 256, 0, a.stream>>>(S, d, list, G.cap, counts, G.gb, bits,
-                                                                         labels, mt, target);
+    k_list_patch<T><<<sm_count() * 8, 256, 0, a.stream>>>(S, d, list, a.counts + a.list_cur, bits, labels, mt, target);
     if (a.launches) *a.launches += 1;
     return cudaGetLastError();
 }
@@ -190,18 +171,18 @@ template <typename T, int NB>
 cudaError_t advect_first_sweep(const BoxSet<T, NB>& S, SweepArgs& a) {
     if (S.n == 0) return cudaSuccess;
     const bool vec = rows_vectorisable(S);
-    const SweepGrid G = sweep_grid(S, vec, a);
-    if ((long long)G.gb * G.cap > a.list_entries || G.gb > kSweepBlocks) return cudaErrorInvalidValue;
+    const int gb = sweep_grid(S, vec, a);
+    if (!lists_fit(S, a)) return cudaErrorInvalidValue;
     unsigned long long* lists[2] = {a.list, a.list + a.list_entries};
-    int* counts[2] = {a.counts, a.counts + kSweepBlocks};
+    int* counts[2] = {a.counts, a.counts + 1};
     const int rot = (int)(a.step % 3), dn = (rot + 1) % 3;
-    launch_list(S, vec, rot, (T)a.tau, lists[0], G.cap, counts[0], G.gb, a.stream);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = scan_face_counts(counts[0], a.offsets, G.gb, a.tile_seg, a.tile_cap, a.stream);
+    cudaError_t e = cudaMemsetAsync(counts[0], 0, sizeof(int), a.stream);
     if (e != cudaSuccess) return e;
-    face_fluxes(S, rot, 0, lists[0], G.cap, G.gb, a);
+    launch_list(S, vec, rot, (T)a.tau, lists[0], counts[0], gb, a.stream);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    return launch_update(S, vec, rot, dn, 0, (T)a.tau, lists[1], G.cap, counts[1], G.gb, a.stream);
+    face_fluxes(S, rot, 0, lists[0], counts[0], counts[1], a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return launch_update(S, vec, rot, dn, 0, (T)a.tau, lists[1], counts[1], gb, a.stream);
 }
 
 }  // namespace vof

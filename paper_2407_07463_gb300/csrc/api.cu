@@ -47,7 +47,6 @@ enum Slot {
     S_MOM,
     S_SHAPE,
     S_NET,
-    S_TILESEG,
     S_COUNT
 };
 
@@ -96,11 +95,10 @@ bool config_valid(const vof_config* c) {
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 size_t nz_map_bytes(size_t words) { return align256(words * sizeof(uint16_t)); }
 
-// Tiles of a face list at its largest (the list's reserved span).
+// Entries of a face list at its largest (the list's reserved span).
 size_t list_entries_for(const vof_config* c) {
-    return (size_t)list_reserve((long long)c->ny * c->nz * ((c->nx + 31) / 32), 1, c->k_capacity);
+    return (size_t)list_reserve((long long)c->ny * c->nz * ((c->nx + 31) / 32), c->k_capacity);
 }
-size_t tile_cap_for(const vof_config* c) { return (list_entries_for(c) + kFaceTile - 1) / kFaceTile; }
 
 Layout layout_for(const vof_config* c) {
     Layout L;
@@ -112,10 +110,9 @@ Layout layout_for(const vof_config* c) {
     L.size[S_BUF1] = K * N * es;
     L.size[S_BUF2] = K * N * es;
     L.size[S_FLUX] = K * N * es;
-    // two face lists segmented by block; a segment holds up to 2 faces per
-    // cell and field of the block's cells, for any grid the advance picks
+    // two face lists
     L.size[S_LIST] = 2 * list_entries_for(c) * 8;
-    L.size[S_COUNTS] = (3 * (size_t)kSweepBlocks + 1) * 4;
+    L.size[S_COUNTS] = 2 * sizeof(int);
     L.size[S_MISC] = kMiscBytes;
     L.size[S_BITS] = K * words * 4;
     L.size[S_CCBITS] = K * words * 4;
@@ -149,8 +146,6 @@ Layout layout_for(const vof_config* c) {
     L.size[S_SHAPE] = (size_t)kDropCap * 7 * 8;
     // network normal at the cell of every listed face (learned normal only)
     L.size[S_NET] = c->precision == VOF_MIXED_LEARNED ? K * N * 16 : 0;
-    // first segment of each tile of kFaceTile entries of a face list
-    L.size[S_TILESEG] = (tile_cap_for(c) + 1) * 4;
     size_t o = 0;
     for (int s = 0; s < S_COUNT; ++s) {
         L.off[s] = o;
@@ -257,6 +252,7 @@ static BoxSet<T, 1> ctx_box_set(vof_ctx* ctx, double* clipped, double dt) {
     B.tile0 = 0;
     B.words = g.rows * g.W;
     B.divW = fastdiv_make((uint32_t)g.W);
+    B.divnx = fastdiv_make((uint32_t)g.nx);
     B.divny = fastdiv_make((uint32_t)g.ny);
     B.sfac = (T)(dt / ctx->cfg.h);
     B.c = (T*)ctx->c;
@@ -463,8 +459,7 @@ vof_status recolour_impl(vof_ctx* ctx, int* moved_out, int* fired_out, SweepArgs
              }));
     ctx->launches += 1;
     if (patch && moved > 0 && ctx->n_active != na0) {
-        // a newly activated field changes the list's segment geometry (its
-        // capacity per segment grows with the fields): list again
+        // a newly activated field joins the maps of non-zero words: list again
         patch->list_valid = false;
     } else if (patch && moved > 0) {
         // the list serves the first sweep of the next step
@@ -661,9 +656,6 @@ vof_status vof_step(vof_ctx* ctx, double dt, int32_t nsteps, vof_step_report* re
     a.list = ctx->slot<unsigned long long>(S_LIST);
     a.list_entries = (long long)list_entries_for(&ctx->cfg);
     a.counts = ctx->slot<int>(S_COUNTS);
-    a.offsets = ctx->slot<int>(S_COUNTS) + 2 * kSweepBlocks;
-    a.tile_seg = ctx->slot<int>(S_TILESEG);
-    a.tile_cap = (int)std::min<size_t>(tile_cap_for(&ctx->cfg), (size_t)INT32_MAX);
     a.tau = occupancy_tau(ctx);
     a.list_valid = false;
     a.list_cur = 0;

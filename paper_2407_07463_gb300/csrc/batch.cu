@@ -49,16 +49,15 @@ bool batch_config_valid(const vof_batch_config* c) {
 // Per-box slices and shared buffers of the batch workspace.
 struct BatchLayout {
     std::vector<size_t> b1, b2, flux, net, ccbits, occbits, nz;
-    size_t nz_maps, nz_bytes, clipped, list, counts, tile_seg, misc, vscan, total;
+    size_t nz_maps, nz_bytes, clipped, list, counts, misc, vscan, total;
     long long list_entries, words;
-    int tile_cap;
 };
 
 BatchLayout batch_layout(const vof_batch_config* cfg, const vof_box_desc* boxes, int n) {
     BatchLayout L;
     const size_t es = cfg->precision == VOF_FP64 ? 8 : 4;
     size_t o = 0;
-    long long words_all = 0, kmax = 1;
+    long long words_all = 0, entries = 0;
     for (int b = 0; b < n; ++b) {
         const vof_box_desc& d = boxes[b];
         const size_t N = (size_t)d.nx * d.ny * d.nz, K = (size_t)d.k_capacity;
@@ -70,7 +69,7 @@ BatchLayout batch_layout(const vof_batch_config* cfg, const vof_box_desc* boxes,
         L.ccbits.push_back(o), o = al256(o + K * words * 4);
         L.occbits.push_back(o), o = al256(o + K * words * 4);
         words_all += (long long)words;
-        kmax = std::max<long long>(kmax, d.k_capacity);
+        entries += list_reserve((long long)words, d.k_capacity);
     }
     // maps of the words that may hold a non-zero value, three per box
     L.nz_maps = o;
@@ -80,12 +79,10 @@ BatchLayout batch_layout(const vof_batch_config* cfg, const vof_box_desc* boxes,
     }
     L.nz_bytes = o - L.nz_maps;
     L.words = words_all;
-    L.list_entries = list_reserve(words_all, n, (int)kmax);
-    L.tile_cap = (int)std::min<long long>((L.list_entries + kFaceTile - 1) / kFaceTile, INT32_MAX);
+    L.list_entries = entries;
     L.clipped = o, o = al256(o + (size_t)n * 16 * 8);
     L.list = o, o = al256(o + 2 * (size_t)L.list_entries * 8);
-    L.counts = o, o = al256(o + (3 * (size_t)kSweepBlocks + 1) * 4);
-    L.tile_seg = o, o = al256(o + ((size_t)L.tile_cap + 1) * 4);
+    L.counts = o, o = al256(o + 2 * sizeof(int));
     L.misc = o, o = al256(o + 64);  // [0] tensor-core status, [8..32) face counters
     L.vscan = o, o = al256(o + 16);
     L.total = o;
@@ -130,6 +127,7 @@ BoxSet<T, kMaxBoxes> batch_set(vof_batch* B) {
         X.tile0 = S.tiles;
         X.words = X.g.rows * X.g.W;
         X.divW = fastdiv_make((uint32_t)X.g.W);
+        X.divnx = fastdiv_make((uint32_t)d.nx);
         X.divny = fastdiv_make((uint32_t)d.ny);
         X.sfac = (T)(d.dt / B->cfg.h);
         X.c = (T*)d.c_dev;
@@ -155,9 +153,6 @@ SweepArgs batch_args(vof_batch* B) {
     a.list = (unsigned long long*)(B->ws + B->L.list);
     a.list_entries = B->L.list_entries;
     a.counts = (int*)(B->ws + B->L.counts);
-    a.offsets = a.counts + 2 * kSweepBlocks;
-    a.tile_seg = (int*)(B->ws + B->L.tile_seg);
-    a.tile_cap = B->L.tile_cap;
     a.step = B->step;
     a.band = B->cfg.alpha_fp64_band;
     // occupancy threshold as in a context: the largest value of the element

@@ -16,7 +16,7 @@
 // output buffer holds.  A tile of up to kTileWords words of one box is the
 // unit of work of a block, which lists the tile's active (word, field) items
 // in shared memory and hands them to its lane groups.
-// The face list of the next sweep holds 64-bit keys box | field | k | j | i.
+// The face list of the next sweep holds 64-bit keys (face_key).
 #pragma once
 
 #include <algorithm>
@@ -59,7 +59,7 @@ struct BoxDev {
     int K;      // fields advected
     int tile0;  // first tile of the box
     int words;  // 32-cell words of one field, rows * W
-    FastDiv divW, divny;  // by W and ny
+    FastDiv divW, divnx, divny;  // by W, nx and ny
     T sfac;     // dt / h
     T* c;       // [K][N] state (updated in place over a step)
     T* b1;      // [K][N] state after the first sweep
@@ -83,11 +83,6 @@ struct BoxSet {
     int tw;     // words per tile, at most kTileWords
     BoxDev<T> b[NB];
 };
-
-// Face-list key: box (6 bits) | field (4) | k | j | i (18 bits each).
-__device__ __forceinline__ unsigned long long box_face_key(int box, int f, int i, int j, int k) {
-    return ((unsigned long long)box << 58) | face_key(f, i, j, k);
-}
 
 template <typename T, int NB>
 __device__ __forceinline__ int box_of_tile(const BoxSet<T, NB>& S, int tile) {
@@ -131,17 +126,14 @@ inline int tile_words(long long words) {
 
 // Place of one word of a tile.
 struct WordPlace {
-    unsigned long long key;   // face key of the word's row (field and i zero)
-    unsigned long long keyn;  // the same of the row one up along dn (dn != 0)
     int x0, i0;               // first cell: index in the field, and along x
     int lo, hi;               // offsets of the neighbour rows along d (d != 0)
     int hin;                  // offset of the high neighbour row along dn (dn != 0)
 };
 
-// Place of word `word` of box `box`, with its neighbour words along d.
+// Place of word `word` of a box, with its neighbour words along d.
 template <typename T>
-__device__ __forceinline__ WordPlace place_word(const BoxDev<T>& B, int box, int word, int d, int dn, int& wlo,
-                                                int& whi) {
+__device__ __forceinline__ WordPlace place_word(const BoxDev<T>& B, int word, int d, int dn, int& wlo, int& whi) {
     const Dims& g = B.g;
     WordPlace p;
     const int row = (int)fastdiv((uint32_t)word, B.divW), wi = word - row * g.W;
@@ -157,14 +149,7 @@ __device__ __forceinline__ WordPlace place_word(const BoxDev<T>& B, int box, int
     wlo = d == 0 ? word + (wi == 0 ? g.W - 1 : -1) : word + rlo * g.W;
     whi = d == 0 ? word + (wi == g.W - 1 ? 1 - g.W : 1) : word + rhi * g.W;
     p.hin = (dn == 1 ? yhi : zhi) * g.nx;
-    p.key = box_face_key(box, 0, 0, j, k);
-    p.keyn = dn == 1 ? box_face_key(box, 0, 0, j == g.ny - 1 ? 0 : j + 1, k)
-                     : box_face_key(box, 0, 0, j, k == g.nz - 1 ? 0 : k + 1);
     return p;
-}
-
-__device__ __forceinline__ unsigned long long key_of(unsigned long long row, int f, int i) {
-    return row | ((unsigned long long)f << 54) | (unsigned long long)i;
 }
 
 // Faces of sweep d whose upwind donor is interfacial, from the state c of
@@ -174,16 +159,14 @@ __device__ __forceinline__ unsigned long long key_of(unsigned long long row, int
 // velocity read once, four fields' loads in flight).
 template <typename T, int NB, int VW>
 __global__ void __launch_bounds__(kSweepThreads) k_list_sp(const __grid_constant__ BoxSet<T, NB> S, int d, T tau,
-                                                           unsigned long long* __restrict__ list, long long cap,
-                                                           int* __restrict__ counts) {
+                                                           unsigned long long* __restrict__ list,
+                                                           int* __restrict__ count) {
     constexpr int LPW = 32 / VW, WPW = 32 / LPW;  // lanes per word, words per warp
     constexpr int FB = 4;                         // fields in flight
-    __shared__ int s_count;
-    if (threadIdx.x == 0) s_count = 0;
-    __syncthreads();
+    __shared__ unsigned long long s_buf[kSweepThreads / 32][kWarpBuf];
     const int lane = threadIdx.x & 31, gl = lane & (LPW - 1);
+    FaceWriter out(s_buf[threadIdx.x >> 5], list, count);
     const unsigned group = (0xffffffffu >> (32 - LPW)) << (lane & ~(LPW - 1));
-    unsigned long long* seg = list + (size_t)blockIdx.x * cap;
     for (int tile = blockIdx.x; tile < S.tiles; tile += gridDim.x) {
         const int bx = box_of_tile(S, tile);
         const BoxDev<T>& B = S.b[bx];
@@ -193,7 +176,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_list_sp(const __grid_constant
             const int word = base + lane / LPW;
             const bool ok = word < w1;
             int wlo, whi;
-            const WordPlace p = place_word(B, bx, ok ? word : w0, d, d, wlo, whi);
+            const WordPlace p = place_word(B, ok ? word : w0, d, d, wlo, whi);
             const bool valid = ok && p.i0 + gl * VW < g.nx;
             const int i = p.i0 + (valid ? gl * VW : 0), x = p.x0 + (valid ? gl * VW : 0);
             // faces of this lane's cells as donors: the low one where the
@@ -242,14 +225,13 @@ __global__ void __launch_bounds__(kSweepThreads) k_list_sp(const __grid_constant
                         const uint32_t fl = inter & nlo, fh = inter & nhi;
                         const int n = __popc(fl) + __popc(fh);
                         if (__any_sync(0xffffffffu, n != 0)) {
-                            int pos = warp_reserve(n, lane, &s_count);
+                            int pos = out.reserve(n, lane);
 #pragma unroll
                             for (int e = 0; e < VW; ++e) {
-                                if ((fl >> e) & 1u) seg[pos++] = key_of(p.key, f, i + e);
-                                if ((fh >> e) & 1u)
-                                    seg[pos++] = d == 0 ? key_of(p.key, f, i + e + 1 == g.nx ? 0 : i + e + 1)
-                                                        : key_of(p.keyn, f, i + e);
+                                if ((fl >> e) & 1u) out.buf[pos++] = face_key(bx, f, 0, x + e);
+                                if ((fh >> e) & 1u) out.buf[pos++] = face_key(bx, f, 1, x + e);
                             }
+                            out.settle(lane);
                         }
                     }
                     if (ok && gl == 0) B.occbits[(size_t)f * B.words + word] = ow;
@@ -258,15 +240,14 @@ __global__ void __launch_bounds__(kSweepThreads) k_list_sp(const __grid_constant
             if (ok && gl == 0) B.nzc[word] = (uint16_t)nz;
         }
     }
-    __syncthreads();
-    if (threadIdx.x == 0) counts[blockIdx.x] = s_count;
+    out.flush(lane);
 }
 
 // Update pass of sweep PH (0, 1, 2) along d (DX: d == 0) for every box:
 // c_out = c_in - (F_hi - F_lo) + c_c (s_hi - s_lo), c_c bits written in
 // sweep 0 and read after, the clip and the occupancy bits in sweep 2, and the
 // faces of the next sweep (direction dn) whose donor is interfacial appended
-// to the block's list segment.
+// to its list.
 //
 // A word of a field is active when it, or a neighbour word along d, may be
 // non-zero in the input, or when the output buffer may hold something there
@@ -283,10 +264,10 @@ __global__ void __launch_bounds__(kSweepThreads) k_list_sp(const __grid_constant
 template <typename T, int NB, int VW, int PH, bool DX>
 __global__ void __launch_bounds__(kSweepThreads, 4)
     k_update_sp(const __grid_constant__ BoxSet<T, NB> S, int d, int dn, T tau,
-                unsigned long long* __restrict__ nlist, long long cap, int* __restrict__ ncounts) {
+                unsigned long long* __restrict__ nlist, int* __restrict__ ncount) {
     constexpr int LPW = 32 / VW, WPW = 32 / LPW;
     constexpr int WARPS = kSweepThreads / 32;
-    __shared__ int s_count;
+    __shared__ unsigned long long s_buf[WARPS][kWarpBuf];
     __shared__ int s_warp[WARPS];
     __shared__ WordPlace s_place[kTileWords];
     __shared__ uint16_t s_item[kTileWords * 16];  // word of the tile << 4 | field
@@ -294,8 +275,7 @@ __global__ void __launch_bounds__(kSweepThreads, 4)
     __shared__ uint32_t s_new[kTileWords];        // fields with a non-zero result
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, gl = lane & (LPW - 1);
     const unsigned group = (0xffffffffu >> (32 - LPW)) << (lane & ~(LPW - 1));
-    if (threadIdx.x == 0) s_count = 0;
-    unsigned long long* seg = nlist + (size_t)blockIdx.x * cap;
+    FaceWriter out(s_buf[warp], nlist, ncount);
     for (int tile = blockIdx.x; tile < S.tiles; tile += gridDim.x) {
         const int bx = box_of_tile(S, tile);
         const BoxDev<T>& B = S.b[bx];
@@ -305,7 +285,7 @@ __global__ void __launch_bounds__(kSweepThreads, 4)
         uint32_t act = 0, out_old = 0;
         if (t0 < nw) {
             int wlo, whi;
-            s_place[t0] = place_word(B, bx, w0 + t0, d, dn, wlo, whi);
+            s_place[t0] = place_word(B, w0 + t0, d, dn, wlo, whi);
             const uint16_t* __restrict__ in = nz_in(B, PH);
             out_old = nz_out(B, PH)[w0 + t0];
             act = ((uint32_t)in[w0 + t0] | in[wlo] | in[whi] | out_old) & ((1u << B.K) - 1u);
@@ -447,14 +427,13 @@ __global__ void __launch_bounds__(kSweepThreads, 4)
             }
             const int nflag = __popc(flo) + __popc(fhi);
             if (__any_sync(0xffffffffu, nflag != 0)) {
-                int pos = warp_reserve(nflag, lane, &s_count);
+                int pos = out.reserve(nflag, lane);
 #pragma unroll
                 for (int e = 0; e < VW; ++e) {
-                    if ((flo >> e) & 1u) seg[pos++] = key_of(p.key, f, i + e);
-                    if ((fhi >> e) & 1u)
-                        seg[pos++] = dn == 0 ? key_of(p.key, f, i + e + 1 == g.nx ? 0 : i + e + 1)
-                                             : key_of(p.keyn, f, i + e);
+                    if ((flo >> e) & 1u) out.buf[pos++] = face_key(bx, f, 0, x + e);
+                    if ((fhi >> e) & 1u) out.buf[pos++] = face_key(bx, f, 1, x + e);
                 }
+                out.settle(lane);
             }
         }
         __syncthreads();
@@ -466,14 +445,13 @@ __global__ void __launch_bounds__(kSweepThreads, 4)
         // (the next tile's first barrier comes before anything reads what its
         // build writes, and this thread's s_new is read above by itself)
     }
-    __syncthreads();
-    if (threadIdx.x == 0) ncounts[blockIdx.x] = s_count;
+    out.flush(lane);
 }
 
 template <typename T, int NB, int VW>
 static void launch_update_vw(const BoxSet<T, NB>& S, int d, int dn, int sweep, T tau, unsigned long long* nlist,
-                             long long cap, int* ncounts, int gb, cudaStream_t st) {
-    auto go = [&](auto kernel) { kernel<<<gb, kSweepThreads, 0, st>>>(S, d, dn, tau, nlist, cap, ncounts); };
+                             int* ncount, int gb, cudaStream_t st) {
+    auto go = [&](auto kernel) { kernel<<<gb, kSweepThreads, 0, st>>>(S, d, dn, tau, nlist, ncount); };
     if (sweep == 0) d == 0 ? go(k_update_sp<T, NB, VW, 0, true>) : go(k_update_sp<T, NB, VW, 0, false>);
     else if (sweep == 1) d == 0 ? go(k_update_sp<T, NB, VW, 1, true>) : go(k_update_sp<T, NB, VW, 1, false>);
     else d == 0 ? go(k_update_sp<T, NB, VW, 2, true>) : go(k_update_sp<T, NB, VW, 2, false>);
@@ -483,21 +461,21 @@ static void launch_update_vw(const BoxSet<T, NB>& S, int d, int dn, int sweep, T
 // cells per lane (whole 16-byte lanes), else one.
 template <typename T, int NB>
 static cudaError_t launch_update(const BoxSet<T, NB>& S, bool vec, int d, int dn, int sweep, T tau,
-                                 unsigned long long* nlist, long long cap, int* ncounts, int gb, cudaStream_t st) {
+                                 unsigned long long* nlist, int* ncount, int gb, cudaStream_t st) {
     if (vec) {
-        launch_update_vw<T, NB, VecOf<T>::W>(S, d, dn, sweep, tau, nlist, cap, ncounts, gb, st);
+        launch_update_vw<T, NB, VecOf<T>::W>(S, d, dn, sweep, tau, nlist, ncount, gb, st);
     } else {
-        if constexpr (NB == 1) launch_update_vw<T, NB, 1>(S, d, dn, sweep, tau, nlist, cap, ncounts, gb, st);
+        if constexpr (NB == 1) launch_update_vw<T, NB, 1>(S, d, dn, sweep, tau, nlist, ncount, gb, st);
     }
     return cudaGetLastError();
 }
 template <typename T, int NB>
-static void launch_list(const BoxSet<T, NB>& S, bool vec, int d, T tau, unsigned long long* list, long long cap,
-                        int* counts, int gb, cudaStream_t st) {
+static void launch_list(const BoxSet<T, NB>& S, bool vec, int d, T tau, unsigned long long* list, int* count, int gb,
+                        cudaStream_t st) {
     if (vec) {
-        k_list_sp<T, NB, VecOf<T>::W><<<gb, kSweepThreads, 0, st>>>(S, d, tau, list, cap, counts);
+        k_list_sp<T, NB, VecOf<T>::W><<<gb, kSweepThreads, 0, st>>>(S, d, tau, list, count);
     } else {
-        if constexpr (NB == 1) k_list_sp<T, NB, 1><<<gb, kSweepThreads, 0, st>>>(S, d, tau, list, cap, counts);
+        if constexpr (NB == 1) k_list_sp<T, NB, 1><<<gb, kSweepThreads, 0, st>>>(S, d, tau, list, count);
     }
 }
 
@@ -513,8 +491,8 @@ static int update_blocks_per_sm() {
     return per_sm;
 }
 
-// A listed face of a box set: box, field, the cell x of the face's high
-// side, the flux index t = f N + x, the upwind donor.
+// A listed face of a box set: box, field, upwind donor, the cell x of the
+// face's high side and the flux index t = f N + x.
 struct BoxFace {
     int box, f, x, donor;
     int di, dj, dk;  // the donor's cell coordinates
@@ -522,28 +500,27 @@ struct BoxFace {
 };
 
 template <typename T, int NB>
-__device__ __forceinline__ BoxFace decode_box_face(const BoxSet<T, NB>& S, unsigned long long key, int d, T& uv) {
+__device__ __forceinline__ BoxFace decode_box_face(const BoxSet<T, NB>& S, unsigned long long key, int d) {
     BoxFace r;
-    r.box = (int)(key >> 58);
-    r.f = (int)((key >> 54) & 15u);
-    const int k = (int)((key >> 36) & 0x3ffffu);
-    const int j = (int)((key >> 18) & 0x3ffffu);
-    const int i = (int)(key & 0x3ffffu);
-    const Dims& g = S.b[r.box].g;
-    r.x = cell(i, j, k, g);
+    r.box = NB == 1 ? 0 : (int)(key >> 36);
+    r.f = (int)((key >> kFaceFieldShift) & 15u);
+    const BoxDev<T>& B = S.b[r.box];
+    const Dims& g = B.g;
+    r.donor = (int)((uint32_t)key & 0x7fffffffu);
+    const int row = (int)fastdiv((uint32_t)r.donor, B.divnx);
+    r.di = r.donor - row * g.nx;
+    r.dk = (int)fastdiv((uint32_t)row, B.divny);
+    r.dj = row - r.dk * g.ny;
+    r.x = r.donor;
+    if ((uint32_t)key >> 31) r.x = step_cell(r.donor, r.di, r.dj, r.dk, d, 1, g);
     r.t = (size_t)r.f * g.N + r.x;
-    uv = S.b[r.box].u[(size_t)d * g.N + r.x];
-    // upwind donor: the face's cell, or its low neighbour along d (periodic)
-    r.di = i;
-    r.dj = j;
-    r.dk = k;
-    if (vsign(uv) > 0) {
-        if (d == 0) r.di = i == 0 ? g.nx - 1 : i - 1;
-        else if (d == 1) r.dj = j == 0 ? g.ny - 1 : j - 1;
-        else r.dk = k == 0 ? g.nz - 1 : k - 1;
-    }
-    r.donor = cell(r.di, r.dj, r.dk, g);
     return r;
+}
+// The face's velocity along d.
+template <typename T, int NB>
+__device__ __forceinline__ T face_velocity(const BoxSet<T, NB>& S, const BoxFace& fc, int d) {
+    const BoxDev<T>& B = S.b[fc.box];
+    return B.u[(size_t)d * B.g.N + fc.x];
 }
 
 // After Step 4 moved drops (one box): every face of the current list (the
@@ -556,35 +533,32 @@ __device__ __forceinline__ BoxFace decode_box_face(const BoxSet<T, NB>& S, unsig
 // donor's tag is read only where the Step 1 snapshot marks it occupied.
 template <typename T>
 __global__ void __launch_bounds__(256) k_list_patch(const __grid_constant__ BoxSet<T, 1> S, int d,
-                                                    unsigned long long* __restrict__ list, long long cap,
-                                                    const int* __restrict__ counts, int nseg,
+                                                    unsigned long long* __restrict__ list,
+                                                    const int* __restrict__ count,
                                                     const uint32_t* __restrict__ bits,
                                                     const int* __restrict__ labels, MoveTables mt,
                                                     const int* __restrict__ target) {
     const Dims& g = S.b[0].g;
     const size_t wpf = (size_t)g.rows * g.W;
-    for (int sg = blockIdx.x; sg < nseg; sg += gridDim.x) {
-        const int n = counts[sg];
-        unsigned long long* seg = list + (size_t)sg * cap;
-        for (int e = threadIdx.x; e < n; e += blockDim.x) {
-            const unsigned long long key = seg[e];
-            const int f = (int)((key >> 54) & 15u);
-            if (mt.mv_count[f] == 0) continue;
-            T uv;
-            const BoxFace fc = decode_box_face(S, key, d, uv);
-            const size_t row = (size_t)fc.dk * g.ny + fc.dj;
-            if (!((bits[(size_t)f * wpf + row * g.W + (fc.di >> 5)] >> (fc.di & 31)) & 1u)) continue;
-            const int l = labels[(size_t)f * g.N + fc.donor];
-            if (!is_moving(mt, f, l)) continue;
-            const int m = moving_index(mt, f, l);
-            const int tg = m >= 0 ? target[m] : -1;
-            if (tg >= 0) seg[e] = (key & ~(15ull << 54)) | ((unsigned long long)tg << 54);
-        }
+    const int n = *count;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+        const unsigned long long key = list[e];
+        const int f = (int)((key >> kFaceFieldShift) & 15u);
+        if (mt.mv_count[f] == 0) continue;
+        const BoxFace fc = decode_box_face(S, key, d);
+        const size_t row = (size_t)fc.dk * g.ny + fc.dj;
+        if (!((bits[(size_t)f * wpf + row * g.W + (fc.di >> 5)] >> (fc.di & 31)) & 1u)) continue;
+        const int l = labels[(size_t)f * g.N + fc.donor];
+        if (!is_moving(mt, f, l)) continue;
+        const int m = moving_index(mt, f, l);
+        const int tg = m >= 0 ? target[m] : -1;
+        if (tg >= 0) list[e] = (key & ~(15ull << kFaceFieldShift)) | ((unsigned long long)tg << kFaceFieldShift);
     }
 }
 
-// MYC fluxes of the listed faces of every box (one thread per face, tiles of
-// kFaceTile consecutive entries whose first segment tile_seg gives).
+// MYC fluxes of the listed faces of every box (one thread per face);
+// *next_count, the count of the list that the sweep's update pass will fill, is
+// set to zero.
 //
 // In double the kernel is bound by FP64 issue (1/64 of the FP32 rate), so
 // its time is its count of FP64 instructions: the forms of plic64.cuh took
@@ -595,15 +569,15 @@ template <typename T, int NB>
 __global__ void __launch_bounds__(kFaceTile) k_face_flux_bx(const __grid_constant__ BoxSet<T, NB> S, int d,
                                                             int sweep, T band,
                                                             const unsigned long long* __restrict__ list,
-                                                            long long cap, const int* __restrict__ off, int nseg,
-                                                            const int* __restrict__ tile_seg) {
-    const int n = off[nseg];
+                                                            const int* __restrict__ count,
+                                                            int* __restrict__ next_count) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *next_count = 0;
+    const int n = *count;
     for (int base = blockIdx.x * kFaceTile; base < n; base += gridDim.x * kFaceTile) {
         const int e = base + threadIdx.x;
         if (e >= n) continue;
-        const int sgi = segment_from(off, tile_seg[base / kFaceTile], e);
-        T uv;
-        const BoxFace fc = decode_box_face(S, list[(size_t)sgi * cap + (e - off[sgi])], d, uv);
+        const BoxFace fc = decode_box_face(S, list[e], d);
+        const T uv = face_velocity(S, fc, d);
         const BoxDev<T>& B = S.b[fc.box];
         T st[27];
         gather_stencil_ijk(sweep_in(B, sweep) + (size_t)fc.f * B.g.N, fc.di, fc.dj, fc.dk, B.g, st);

@@ -51,12 +51,14 @@ __device__ __forceinline__ int cell(int i, int j, int k, const Dims& g) {
     return (k * g.ny + j) * g.nx + i;
 }
 
-// Face-list entry: the face is the low face (along a sweep) of cell
-// (i, j, k) of field f, packed so that decoding needs no division.
-__device__ __forceinline__ unsigned long long face_key(int f, int i, int j, int k) {
-    return ((unsigned long long)f << 54) | ((unsigned long long)k << 36) | ((unsigned long long)j << 18) |
-           (unsigned long long)i;
+// Face-list entry: box (6 bits) | field (4) | side (1) | upwind donor cell
+// (31); the face is the donor's low (side 0) or high (side 1) face along the
+// sweep, so that the donor's stencil can be fetched before the velocity.
+__device__ __forceinline__ unsigned long long face_key(int box, int f, int side, int donor) {
+    return ((unsigned long long)box << 36) | ((unsigned long long)f << 32) |
+           (unsigned long long)((uint32_t)side << 31 | (uint32_t)donor);
 }
+constexpr int kFaceFieldShift = 32;
 
 // Neighbour of x one cell along axis d in direction dir (+1/-1), periodic.
 __device__ __forceinline__ int step_cell(int x, int i, int j, int k, int d, int dir, const Dims& g) {

@@ -39,34 +39,31 @@ static_assert(kFaceTile == 128, "one face per thread of a 128-thread CTA");
 template <int NB>
 __global__ void __launch_bounds__(128, 4) k_face_normals_net(const __grid_constant__ BoxSet<float, NB> S, int d,
                                                              int sweep, const unsigned long long* __restrict__ list,
-                                                             long long cap, const int* __restrict__ off,
-                                                             int nseg, const int* __restrict__ tile_seg,
+                                                             const int* __restrict__ count,
+                                                             int* __restrict__ next_count,
                                                              const MlpBlob* __restrict__ w,
                                                              int* __restrict__ status) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     MlpSmem& s = *reinterpret_cast<MlpSmem*>(smem_raw);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *next_count = 0;
     mlp_cta_begin(s, w);
     const uint32_t taddr = s.tbase;
     uint32_t phase = 0;
     const int t = threadIdx.x;
-    const int n = off[nseg];
+    const int n = *count;
     const int stride = gridDim.x * 128;
     // The stencils of the next tile are gathered while this tile's layers run
-    // (27 registers), the key of the one after that while they are: the three
-    // dependent loads of a face (key, velocity, stencil) leave the critical
-    // path.  256^3, K = 8: 0.29 ms per sweep against 0.31 gathering first.
+    // (27 registers), the key of the one after that while they are: the
+    // dependent loads of a face (key, stencil) leave the critical
+    // path.  256^3, K = 8: 0.27 ms per sweep against 0.31 gathering first.
     auto load_key = [&](int base) -> unsigned long long {
-        const int e = base + t;
-        if (e >= n) return 0ull;
-        const int sgi = segment_from(off, tile_seg[base / kFaceTile], e);
-        return list[(size_t)sgi * cap + (e - off[sgi])];
+        return base + t < n ? list[base + t] : 0ull;
     };
     float st[27];
     float4* dst = nullptr;
     auto gather = [&](int base, unsigned long long key) {
         if (base + t < n) {
-            float uv;
-            const BoxFace fc = decode_box_face(S, key, d, uv);
+            const BoxFace fc = decode_box_face(S, key, d);
             const BoxDev<float>& B = S.b[fc.box];
             dst = B.net + fc.t;
             gather_stencil_ijk(sweep_in(B, sweep) + (size_t)fc.f * B.g.N, fc.di, fc.dj, fc.dk, B.g, st);
@@ -115,11 +112,10 @@ __global__ void __launch_bounds__(128, 4) k_face_normals_net(const __grid_consta
 constexpr int kJudgeTile = 128, kJudgeWarps = kJudgeTile / 32;
 
 template <int NB>
-__global__ void __launch_bounds__(kJudgeTile) k_face_flux_judged(const __grid_constant__ BoxSet<float, NB> S, int d,
+__global__ void __launch_bounds__(kJudgeTile, 8) k_face_flux_judged(const __grid_constant__ BoxSet<float, NB> S, int d,
                                                           int sweep, float band,
                                                           const unsigned long long* __restrict__ list,
-                                                          long long cap, const int* __restrict__ off, int nseg,
-                                                          const int* __restrict__ tile_seg, float tol,
+                                                          const int* __restrict__ count, float tol,
                                                           unsigned long long* __restrict__ counters) {
     __shared__ float s_st[27][kJudgeTile];  // stencil of thread t's donor in column t
     __shared__ float s_m[4][kJudgeTile];    // MYC's normal and plane constant where it replaces the network's
@@ -128,20 +124,23 @@ __global__ void __launch_bounds__(kJudgeTile) k_face_flux_judged(const __grid_co
     __shared__ unsigned char s_myc[kJudgeTile];
     __shared__ int s_wq[kJudgeWarps];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int n = off[nseg];
+    const int n = *count;
     unsigned n_net = 0, n_myc = 0, n_queued = 0;
+    // the key of this thread's face, loaded a tile ahead
+    auto load_key = [&](int base) -> unsigned long long {
+        return base + t < n ? list[base + t] : 0ull;
+    };
+    unsigned long long next = load_key(blockIdx.x * kJudgeTile);
     for (int base = blockIdx.x * kJudgeTile; base < n; base += gridDim.x * kJudgeTile) {
-        const int e = base + t;
-        const bool valid = e < n;
+        const unsigned long long key = next;
+        const bool valid = base + t < n;
         float sv = 0.f, mn[3] = {1.f, 0.f, 0.f};
         bool net_ok = false;
         float* dst = nullptr;
         if (valid) {
-            const int sgi = segment_from(off, tile_seg[base / kFaceTile], e);
-            float uv;
-            const BoxFace fc = decode_box_face(S, list[(size_t)sgi * cap + (e - off[sgi])], d, uv);
+            const BoxFace fc = decode_box_face(S, key, d);
             const BoxDev<float>& B = S.b[fc.box];
-            sv = uv * B.sfac;
+            sv = face_velocity(S, fc, d) * B.sfac;
             dst = B.flux + fc.t;
             float st[27];
             gather_stencil_ijk(sweep_in(B, sweep) + (size_t)fc.f * B.g.N, fc.di, fc.dj, fc.dk, B.g, st);
@@ -152,6 +151,7 @@ __global__ void __launch_bounds__(kJudgeTile) k_face_flux_judged(const __grid_co
             net_ok = l1_normalise(nn, mn);
         }
         s_myc[t] = 0;
+        next = load_key(base + gridDim.x * kJudgeTile);
         __syncthreads();
         // network residual of every face; the ones above the tolerance queue,
         // in face order (a thread then reads the stencil column of its own
@@ -255,33 +255,29 @@ __global__ void __launch_bounds__(kJudgeTile) k_face_flux_judged(const __grid_co
 }
 
 template <int NB>
-void face_normals_net_set(const BoxSet<float, NB>& S, int d, int sweep, const unsigned long long* list, long long cap,
-                          const int* off, int nseg, const int* tile_seg, const MlpBlob* w, int* status,
-                          cudaStream_t st) {
+void face_normals_net_set(const BoxSet<float, NB>& S, int d, int sweep, const unsigned long long* list,
+                          const int* count, int* next_count, const MlpBlob* w, int* status, cudaStream_t st) {
     static bool attr = false;
     if (!attr) {
         cudaFuncSetAttribute(k_face_normals_net<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)sizeof(MlpSmem));
         attr = true;
     }
-    k_face_normals_net<NB><<<sm_count() * 4, 128, sizeof(MlpSmem), st>>>(S, d, sweep, list, cap, off, nseg, tile_seg, w,
-                                                                  status);
+    k_face_normals_net<NB><<<sm_count() * 4, 128, sizeof(MlpSmem), st>>>(S, d, sweep, list, count, next_count, w,
+                                                                         status);
 }
 
 template <int NB>
 void face_flux_judged_set(const BoxSet<float, NB>& S, int d, int sweep, float band, const unsigned long long* list,
-                          long long cap, const int* off, int nseg, const int* tile_seg, float tol,
-                          unsigned long long* counters, cudaStream_t st) {
-    k_face_flux_judged<NB><<<sm_count() * (16 * 128 / kJudgeTile), kJudgeTile, 0, st>>>(S, d, sweep, band, list, cap, off, nseg, tile_seg, tol, counters);
+                          const int* count, float tol, unsigned long long* counters, cudaStream_t st) {
+    k_face_flux_judged<NB><<<sm_count() * (16 * 128 / kJudgeTile), kJudgeTile, 0, st>>>(S, d, sweep, band, list, count, tol, counters);
 }
 
-#define VOF_LEARNED_SET(NB)                                                                                       \
-    template void face_normals_net_set<NB>(const BoxSet<float, NB>&, int, int, const unsigned long long*,         \
-                                           long long, const int*, int, const int*, const MlpBlob*, int*,          \
-                                           cudaStream_t);                                                         \
-    template void face_flux_judged_set<NB>(const BoxSet<float, NB>&, int, int, float, const unsigned long long*,  \
-                                           long long, const int*, int, const int*, float, unsigned long long*,    \
-                                           cudaStream_t);
+#define VOF_LEARNED_SET(NB)                                                                                      \
+    template void face_normals_net_set<NB>(const BoxSet<float, NB>&, int, int, const unsigned long long*,        \
+                                           const int*, int*, const MlpBlob*, int*, cudaStream_t);                \
+    template void face_flux_judged_set<NB>(const BoxSet<float, NB>&, int, int, float, const unsigned long long*, \
+                                           const int*, float, unsigned long long*, cudaStream_t);
 VOF_LEARNED_SET(1)
 VOF_LEARNED_SET(kMaxBoxes)
 #undef VOF_LEARNED_SET

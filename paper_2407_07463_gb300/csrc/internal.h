@@ -54,7 +54,6 @@ constexpr unsigned long long kEmptyKey = ~0ull;
 constexpr int kPairCap = 1 << 16;     // distinct tagged near-contact pairs per call
 constexpr int kMoveCap = 2048;        // moving drops per recolour call
 constexpr int kDropCap = 1 << 20;     // drops over all fields for statistics
-constexpr int kSweepBlocks = 152 * 64; // most blocks (and face-list segments) of a sweep (buffer capacity)
 
 // Keeps the name of the last CUDA error a library call met (for
 // vof_last_cuda_error); returns the error unchanged.
@@ -67,16 +66,15 @@ template <typename T, int NB>
 struct BoxSet;
 constexpr int kMaxBoxes = 64;
 // Learned normal of a box set (FP32 path): network normals of the listed
-// faces of one sweep (tensor cores), then their judged fluxes;
+// faces of one sweep (tensor cores; *next_count, the count of the list that
+// the sweep's update pass will fill, set to zero), then their judged fluxes;
 // counters[0/1] += faces on the network's / MYC's normal.
 template <int NB>
-void face_normals_net_set(const BoxSet<float, NB>& S, int d, int sweep, const unsigned long long* list, long long cap,
-                          const int* off, int nseg, const int* tile_seg, const MlpBlob* w, int* status,
-                          cudaStream_t st);
+void face_normals_net_set(const BoxSet<float, NB>& S, int d, int sweep, const unsigned long long* list,
+                          const int* count, int* next_count, const MlpBlob* w, int* status, cudaStream_t st);
 template <int NB>
 void face_flux_judged_set(const BoxSet<float, NB>& S, int d, int sweep, float band, const unsigned long long* list,
-                          long long cap, const int* off, int nseg, const int* tile_seg, float tol,
-                          unsigned long long* counters, cudaStream_t st);
+                          const int* count, float tol, unsigned long long* counters, cudaStream_t st);
 // nsteps steps of every box of a set (one box: a context; up to kMaxBoxes:
 // a batch).
 cudaError_t advect_set_fp64(const BoxSet<double, 1>& S, SweepArgs& a, int nsteps);
@@ -98,21 +96,12 @@ int update_occupancy_fp64();
 // Listing and first sweep of a batch only (state untouched; for timing).
 cudaError_t advect_first_sweep_fp64(const BoxSet<double, kMaxBoxes>& S, SweepArgs& a);
 cudaError_t advect_first_sweep_fp32(const BoxSet<float, kMaxBoxes>& S, SweepArgs& a);
-// Face-list entries to reserve per list for up to K fields of n_boxes boxes
-// of `words` 32-cell words in all: up to 2 faces per cell of every word of
-// the blocks' tiles, a last tile per box and at least 64 blocks (sweep_grid).
-inline long long list_reserve(long long words, int n_boxes, int K) {
-    const long long padded = words + 128LL * n_boxes;
-    return 64LL * K * (padded + padded / 64 + 256);
-}
+// Face-list entries to reserve per list for K fields of `words` 32-cell
+// words: up to 2 faces per cell.
+inline long long list_reserve(long long words, int K) { return 64LL * K * words; }
 
-// Exclusive scan of n ints (one block); off[n] = total.
-cudaError_t scan_counts(const int* counts, int* off, int n, cudaStream_t st);
 // Face lists: consumers take tiles of kFaceTile consecutive entries.
 constexpr int kFaceTile = 128;
-// Exclusive scan of the segment lengths of a face list, plus tile_seg[t] =
-// the segment holding entry t * kFaceTile (t < tile_cap).
-cudaError_t scan_face_counts(const int* counts, int* off, int n, int* tile_seg, int tile_cap, cudaStream_t st);
 cudaError_t pack_bits(const void* c, bool fp64, uint32_t* bits, const Dims& g, int K, double tau,
                       cudaStream_t st);
 // Box dilation (Chebyshev distance reach, periodic) of n bit planes from src
