@@ -85,31 +85,16 @@ __device__ __forceinline__ void canon_output(const float nc[3], const CanonFrame
     }
 }
 
-// BF16 split of a layer input: x ~ hi + lo with both parts representable
-// (about 16 significant bits; each weight multiplies both parts).
-__device__ __forceinline__ void split_bf16(float x, __nv_bfloat16& hi, __nv_bfloat16& lo) {
-    hi = __float2bfloat16_rn(x);
-    lo = __float2bfloat16_rn(x - __bfloat162float(hi));
-}
-
-// Store v as the pair (hi at column k, lo at column k + half) of row r of a
-// K-major tile with kext columns.
-__device__ __forceinline__ void store_pair(unsigned char* tile, int r, int k, int half, int kext, float v) {
-    __nv_bfloat16 hi, lo;
-    split_bf16(v, hi, lo);
-    *reinterpret_cast<__nv_bfloat16*>(tile + tc::kmajor_offset(r, k, kext)) = hi;
-    *reinterpret_cast<__nv_bfloat16*>(tile + tc::kmajor_offset(r, k + half, kext)) = lo;
-}
-
 // Eight consecutive layer inputs v[0..7] of row r (columns k0..k0+7, k0 a
-// multiple of 8) as pairs: one 16-byte store of the high parts at column k0
+// multiple of 8) as BF16 pairs, x ~ hi + lo (about 16 significant bits; each
+// weight multiplies both parts): one 16-byte store of the high parts at column k0
 // and one of the low parts at column k0 + half (a core-matrix row holds 8
 // consecutive K elements).
 __device__ __forceinline__ void store_pairs8(unsigned char* tile, int r, int k0, int half, int kext, const float v[8]) {
     uint32_t hi[4], lo[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        // split_bf16 on two values at once: one packed conversion per part
+        // x ~ hi + lo on two values at once: one packed conversion per part
         const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
         // v - hi for both in one packed operation (exact product by -1)
         const float2 r = __ffma2_rn(__bfloat1622float2(h), make_float2(-1.f, -1.f), make_float2(v[2 * q], v[2 * q + 1]));
@@ -136,17 +121,6 @@ __device__ __forceinline__ void canon_input_col(const float* col, int stride, co
 #pragma unroll
             for (int ic = -1; ic <= 1; ++ic)
                 x[(kc + 1) * 9 + (jc + 1) * 3 + (ic + 1)] = col[(13 + ic * s[0] + jc * s[1] + kc * s[2]) * stride] - 0.5f;
-}
-
-// Weight matrix w[rows][cols] (global, BF16) into a K-major tile holding it
-// twice along K: columns c and cols + c.
-__device__ __forceinline__ void load_weight_pair(unsigned char* tile, const __nv_bfloat16* __restrict__ w, int rows,
-                                                 int cols, int tid, int nthreads) {
-    for (int idx = tid; idx < rows * cols; idx += nthreads) {
-        const int o = idx / cols, i = idx % cols;
-        *reinterpret_cast<__nv_bfloat16*>(tile + tc::kmajor_offset(o, i, 2 * cols)) = w[idx];
-        *reinterpret_cast<__nv_bfloat16*>(tile + tc::kmajor_offset(o, cols + i, 2 * cols)) = w[idx];
-    }
 }
 
 }  // namespace vof
