@@ -565,30 +565,68 @@ __global__ void __launch_bounds__(256) k_list_patch(const __grid_constant__ BoxS
 // it from 6.2 to 1.5 ms per sweep of the 256^3, K = 8, phi = 0.3 box (2.7 M
 // faces), and a sweep of 32^3 with 8 drops, where one warp's chain is the
 // time, from 78 to 28 us with its other launches.
+//
+// In FP32 the faces whose fraction lies within `band` of 0 or 1 (one in six)
+// take an FP64 step: they are compacted to the first threads of the block, so
+// that one warp in four issues it (the FP64 pipe was 57 to 69% busy with every
+// warp doing so: 66 -> MIXFIG us per sweep at 192 x 160 x 224, K = 6).
 template <typename T, int NB>
 __global__ void __launch_bounds__(kFaceTile) k_face_flux_bx(const __grid_constant__ BoxSet<T, NB> S, int d,
                                                             int sweep, T band,
                                                             const unsigned long long* __restrict__ list,
                                                             const int* __restrict__ count,
                                                             int* __restrict__ next_count) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) *next_count = 0;
+    constexpr bool kBanded = std::is_same<T, float>::value;
+    constexpr int kWarps = kFaceTile / 32;
+    __shared__ T s_q[kBanded ? 4 : 1][kBanded ? kFaceTile : 1];  // queued normals and fractions, then constants
+    __shared__ int s_n[kWarps];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    if (blockIdx.x == 0 && t == 0) *next_count = 0;
     const int n = *count;
     for (int base = blockIdx.x * kFaceTile; base < n; base += gridDim.x * kFaceTile) {
-        const int e = base + threadIdx.x;
-        if (e >= n) continue;
-        const BoxFace fc = decode_box_face(S, list[e], d);
-        const T uv = face_velocity(S, fc, d);
-        const BoxDev<T>& B = S.b[fc.box];
-        T st[27];
-        gather_stencil_ijk(sweep_in(B, sweep) + (size_t)fc.f * B.g.N, fc.di, fc.dj, fc.dk, B.g, st);
-        T m[3];
-        if constexpr (std::is_same<T, double>::value) {
-            myc_direction64(st, m);
-            B.flux[fc.t] = face_flux64(m, st[13], d, uv * B.sfac);
-        } else {
-            myc_normal(st, m);
-            const T alpha = plic_alpha_banded(m[0], m[1], m[2], st[13], band);
-            B.flux[fc.t] = face_flux(m, alpha, d, uv * B.sfac);
+        const bool valid = base + t < n;
+        T m[3] = {T(1), T(0), T(0)}, cv = T(0.5), sv = T(0);
+        T* dst = nullptr;
+        if (valid) {
+            const BoxFace fc = decode_box_face(S, list[base + t], d);
+            const BoxDev<T>& B = S.b[fc.box];
+            sv = face_velocity(S, fc, d) * B.sfac;
+            dst = B.flux + fc.t;
+            T st[27];
+            gather_stencil_ijk(sweep_in(B, sweep) + (size_t)fc.f * B.g.N, fc.di, fc.dj, fc.dk, B.g, st);
+            cv = st[13];
+            if constexpr (kBanded) {
+                myc_normal(st, m);
+            } else {
+                myc_direction64(st, m);
+                *dst = face_flux64(m, cv, d, sv);
+            }
+        }
+        if constexpr (kBanded) {
+            const bool queue = valid && (cv < band || cv > T(1) - band);
+            const unsigned vote = __ballot_sync(0xffffffffu, queue);
+            if (lane == 0) s_n[warp] = __popc(vote);
+            __syncthreads();
+            int at = __popc(vote & ((1u << lane) - 1u)), nq = 0;
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) {
+                at += w < warp ? s_n[w] : 0;
+                nq += s_n[w];
+            }
+            if (queue) {
+                s_q[0][at] = m[0];
+                s_q[1][at] = m[1];
+                s_q[2][at] = m[2];
+                s_q[3][at] = cv;
+            }
+            __syncthreads();
+            if (t < nq) s_q[3][t] = plic_alpha_banded(s_q[0][t], s_q[1][t], s_q[2][t], s_q[3][t], band);
+            T alpha = T(0);
+            if (valid && !queue) alpha = plic_alpha<T>(m[0], m[1], m[2], cv);
+            __syncthreads();
+            if (queue) alpha = s_q[3][at];
+            if (valid) *dst = face_flux(m, alpha, d, sv);
+            // (s_q is written again only after the next tile's first barrier)
         }
     }
 }
