@@ -62,16 +62,14 @@ inline bool rows_vectorisable(const BoxSet<T, NB>& S) {
     return B.g.nx % VecOf<T>::W == 0 && (((uintptr_t)B.c | (uintptr_t)B.u) & 15) == 0;
 }
 
-// Blocks of a list-writing pass: every block takes the same number of tiles
-// (up to the last block's rest), the fewest that the resident blocks can
-// share out.
+// Blocks of a list-writing pass: what the GPU holds at once, the tiles dealt
+// out in turn (equal numbers of tiles per block, with fewer blocks, left SMs
+// with three blocks beside SMs with four: 5 to 20% of the pass).
 template <typename T, int NB>
 int sweep_grid(const BoxSet<T, NB>& S, bool vec, const SweepArgs& a) {
     int per_sm = a.update_blocks_per_sm;
     if (per_sm <= 0) per_sm = std::max(1, vec ? update_blocks_per_sm<T, NB, VecOf<T>::W>() : update_blocks_per_sm<T, NB, 1>());
-    const int most = sm_count() * per_sm;
-    const int per_block = (S.tiles + most - 1) / most;
-    return (S.tiles + per_block - 1) / per_block;
+    return std::min(S.tiles, sm_count() * per_sm);
 }
 
 // Whether the reserved lists hold every face the set can list.

@@ -259,8 +259,8 @@ __global__ void __launch_bounds__(kSweepThreads) k_list_sp(const __grid_constant
 // its velocities come from L1 after the first.
 //
 // Bound: latency (three dependent loads per item: map, values, listed flux).
-// 256^3, K = 8, phi = 0.3, FP32: 0.19 ms per y or z sweep (0.38 ms when every
-// word of every field was read and written), 0.31 ms per x sweep (0.43 ms).
+// 256^3, K = 8, phi = 0.3, FP32: 0.17 ms per y or z sweep (0.38 ms when every
+// word of every field was read and written), 0.28 ms per x sweep (0.43 ms).
 template <typename T, int NB, int VW, int PH, bool DX>
 __global__ void __launch_bounds__(kSweepThreads, 4)
     k_update_sp(const __grid_constant__ BoxSet<T, NB> S, int d, int dn, T tau,
@@ -374,23 +374,39 @@ __global__ void __launch_bounds__(kSweepThreads, 4)
             uint32_t flo = 0, fhi = 0, occm = 0;
             bool nonzero = false, clipped = false;
             const T* __restrict__ flux = B.flux + (size_t)f * g.N;
+            // upwind donors through the low and high faces: empty (no flux),
+            // full (flux s) or interfacial (the listed flux)
+            bool change[VW], full_lo[VW], full_hi[VW];
+            T F_lo[VW], F_hi[VW];
+            bool any = false;
 #pragma unroll
             for (int e = 0; e < VW; ++e) {
-                // upwind donors through the low and high faces: empty (no
-                // flux), full (flux s) or interfacial (the listed flux)
                 const int sl = vsign(ulo[e]), sh = vsign(uhi[e]);
                 const T dl = sl > 0 ? cl[e] : cx[e], dh = sh < 0 ? ch[e] : cx[e];
                 const bool ml = valid && sl != 0 && above_zero(dl), mh = valid && sh != 0 && above_zero(dh);
-                const bool cc = (ccm >> e) & 1u;
+                full_lo[e] = ml && at_least_one(dl);
+                full_hi[e] = mh && at_least_one(dh);
+                F_lo[e] = F_hi[e] = T(0);
+                if (ml && !full_lo[e]) F_lo[e] = flux[x + e];
+                if (mh && !full_hi[e]) F_hi[e] = flux[DX ? (e < VW - 1 ? x + e + 1 : xn) : x + e + hi];
+                change[e] = ml || mh || ((ccm >> e) & 1u);
+                any = any || change[e];
                 v[e] = cx[e];
-                if (ml || mh || cc) {
+            }
+            // the arithmetic once for the warp, its cases by selects (branches
+            // ran it with four lanes at a time: in double the FP64 pipe was
+            // 79% busy at a tenth of its lanes)
+            if (__any_sync(0xffffffffu, any)) {
+#pragma unroll
+                for (int e = 0; e < VW; ++e) {
                     const T s_lo = mul_rn(ulo[e], B.sfac), s_hi = mul_rn(uhi[e], B.sfac);
-                    T F_lo = T(0), F_hi = T(0);
-                    if (ml) F_lo = at_least_one(dl) ? s_lo : flux[x + e];
-                    if (mh) F_hi = at_least_one(dh) ? s_hi : flux[DX ? (e < VW - 1 ? x + e + 1 : xn) : x + e + hi];
-                    v[e] = cx[e] - (F_hi - F_lo);
-                    if (cc) v[e] += s_hi - s_lo;
+                    const T lo = full_lo[e] ? s_lo : F_lo[e], hi_ = full_hi[e] ? s_hi : F_hi[e];
+                    const T r = cx[e] - (hi_ - lo), rc = r + (s_hi - s_lo);
+                    if (change[e]) v[e] = (ccm >> e) & 1u ? rc : r;
                 }
+            }
+#pragma unroll
+            for (int e = 0; e < VW; ++e) {
                 rem[e] = T(0);
                 if (PH == 2) {
                     const bool under = below_zero(v[e]), over = above(v[e], T(1));
@@ -562,14 +578,14 @@ __global__ void __launch_bounds__(256) k_list_patch(const __grid_constant__ BoxS
 //
 // In double the kernel is bound by FP64 issue (1/64 of the FP32 rate), so
 // its time is its count of FP64 instructions: the forms of plic64.cuh took
-// it from 6.2 to 1.5 ms per sweep of the 256^3, K = 8, phi = 0.3 box (2.7 M
+// it from 6.2 to 1.08 ms per sweep of the 256^3, K = 8, phi = 0.3 box (2.7 M
 // faces), and a sweep of 32^3 with 8 drops, where one warp's chain is the
-// time, from 78 to 28 us with its other launches.
+// time, from 78 to 22 us with its other launches.
 //
 // In FP32 the faces whose fraction lies within `band` of 0 or 1 (one in six)
 // take an FP64 step: they are compacted to the first threads of the block, so
 // that one warp in four issues it (the FP64 pipe was 57 to 69% busy with every
-// warp doing so: 66 -> MIXFIG us per sweep at 192 x 160 x 224, K = 6).
+// warp doing so: 66 -> 56 us per sweep at 192 x 160 x 224, K = 6).
 template <typename T, int NB>
 __global__ void __launch_bounds__(kFaceTile) k_face_flux_bx(const __grid_constant__ BoxSet<T, NB> S, int d,
                                                             int sweep, T band,

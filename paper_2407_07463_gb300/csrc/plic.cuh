@@ -185,7 +185,7 @@ __device__ __forceinline__ float alpha_pw(const VolPW& p, float cv) {
 // the components that occur in a step), for the FP64 forms' products.
 __device__ __forceinline__ double scale64(double c) {
     const int e = (int)(bits64(c) >> 52) - 1023;
-    if (e > -256 && e < 256) return 1.0;
+    if (e > -20 && e < 20) return 1.0;
     return from_bits64((long long)(1023 - max(-1000, min(1000, e))) << 52);
 }
 
@@ -387,7 +387,8 @@ __device__ __forceinline__ void myc_normal(const T* st, T m[3]) {
 }
 
 __device__ __forceinline__ void myc_normal(const double* st, double m[3]) {
-    const double il = 1.0 / myc_direction64(st, m);
+    myc_direction64(st, m);
+    const double il = 1.0 / (fabs(m[0]) + fabs(m[1]) + fabs(m[2]));
     m[0] *= il;
     m[1] *= il;
     m[2] *= il;

@@ -85,28 +85,35 @@ VOF_HD double cbrt64(double t) {
 }
 
 // Volume under the plane a x + b y + c z < x in the unit cube, sorted
-// 0 <= a <= b <= c, c > 0, 0 <= x <= (a + b + c) / 2.
-VOF_HD double vol64_half(double a, double b, double c, double x) {
+// 0 <= a <= b <= c, c > 0, 0 <= x <= (a + b + c) / 2, by its piece.
+enum VolPiece { kVolTip = 0, kVolPrism = 1, kVolEdge = 2, kVolCorner = 3 };
+VOF_HD int vol64_piece(double a, double b, double c, double x) {
+    if (le_pos(x, a)) return kVolTip;
+    if (lt_pos(a + b, x)) return kVolPrism;  // (x <= S/2 leaves it to c > a + b)
+    return le_pos(x, b) ? kVolEdge : kVolCorner;
+}
+VOF_HD double vol64_of(int piece, double a, double b, double c, double x) {
     double num, den;
-    if (le_pos(x, a)) {
+    if (piece == kVolTip) {
         num = x * x * x;
         den = 6.0 * a * b * c;
-    } else if (lt_pos(a + b, x)) {  // the prism (x <= S/2 leaves it to c > a + b)
+    } else if (piece == kVolPrism) {
         num = fma(2.0, x, -(a + b));
         den = 2.0 * c;
     } else {
-        const double q = fma(3.0 * x, x - a, a * a);
-        const double tb = x - b;
+        num = fma(3.0 * x, x - a, a * a);
         den = 6.0 * b * c;
-        num = q;
-        if (bits64(tb) > 0) {  // not at x = b, where a may be zero
-            const double tc = plus64(x - c);
-            num = fma(a, q, -fma(tb * tb, tb, tc * tc * tc));
+        if (piece == kVolCorner) {
+            const double tb = x - b, tc = plus64(x - c);
+            num = fma(a, num, -fma(tb * tb, tb, tc * tc * tc));
             den *= a;
         }
     }
     // a divisor this small belongs to a plane whose volume is below 1e-90
     return lt_pos(den, 1e-290) ? 0.0 : num / den;
+}
+VOF_HD double vol64_half(double a, double b, double c, double x) {
+    return vol64_of(vol64_piece(a, b, c, x), a, b, c, x);
 }
 
 // The same for any x; S = a + b + c > 0.
@@ -125,20 +132,43 @@ VOF_HD double vol64(double a, double b, double c, double x) {
 //   c >= a + b, 2w >= 1 + p:  the prism, x = w + (1 + p)/2
 //   else  p (3x(x - p) + p^2 - 6w) = (x - 1)^3 + (x - g)_+^3, seeded by the
 //   middle root of the cubic in trigonometric form (alpha_sorted_pw).
-VOF_HD double alpha64_half(double a, double b, double c, double v) {
-    if (lt_pos(b, 1e-30 * c)) return c * v;  // a plane across one axis (off by < 1e-30 c)
-    const double cv = c * v, ib = 1.0 / b;
-    const double p = a * ib, w6 = 6.0 * cv * ib, p2 = p * p;
-    if (le_pos(w6, p2)) return b * cbrt64(p * w6);
-    if (!negative64(fma(3.0, 1.0 - p, p2) - w6))
-        return b * (0.5 * (p + sqrt(fma(-1.0 / 3.0, p2, (4.0 / 3.0) * w6))));
+enum AlphaPiece { kAlphaLinear = 0, kAlphaCbrt = 1, kAlphaSqrt = 2, kAlphaCubic = 3 };
+// 1 / b for b within FP32's range: two Newton steps from the FP32 quotient.
+VOF_HD double rcp64(double b) {
+    double r = (double)(1.f / (float)b);
+    r = fma(fma(-b, r, 1.0), r, r);
+    return fma(fma(-b, r, 1.0), r, r);
+}
+// The piece the root lies in and its scaled variables p, w6 = 6w and g (g only
+// for the cubic); the linear pieces' root in x.  c within 2^-20 .. 2^20.
+VOF_HD int alpha64_piece(double a, double b, double c, double v, double& p, double& w6, double& g, double& x) {
+    const double cv = c * v;
+    x = cv;
+    if (lt_pos(b, 1e-30 * c)) return kAlphaLinear;  // a plane across one axis (off by < 1e-30 c)
+    const double ib = rcp64(b);
+    p = a * ib;
+    w6 = 6.0 * cv * ib;
+    const double p2 = p * p;
+    if (le_pos(w6, p2)) return kAlphaCbrt;
+    if (!negative64(fma(3.0, 1.0 - p, p2) - w6)) return kAlphaSqrt;
     const double ab = a + b;
-    const bool prism = le_pos(ab, c);
-    if (prism && le_pos(ab, 2.0 * cv)) return fma(0.5, ab, cv);
-    const double g = c * ib;
-    const double hi = prism ? 1.0 + p : 0.5 * (1.0 + p + g);
+    if (le_pos(ab, c) && le_pos(ab, 2.0 * cv)) {
+        x = fma(0.5, ab, cv);
+        return kAlphaLinear;
+    }
+    g = c * ib;
+    return kAlphaCubic;
+}
+VOF_HD double alpha64_cbrt(double p, double w6, double b) { return b * cbrt64(p * w6); }
+VOF_HD double alpha64_sqrt(double p, double w6, double b) {
+    return b * (0.5 * (p + sqrt(fma(-1.0 / 3.0, p * p, (4.0 / 3.0) * w6))));
+}
+VOF_HD double alpha64_cubic(double p, double w6, double g, double b) {
     // seed
     const float pf = (float)p, gf = (float)g, wf = (float)w6 * (1.f / 6.f);
+    const double p1 = 1.0 + p;
+    const bool prism = le_pos(p1, g);
+    const double hi = prism ? p1 : 0.5 * (p1 + g);
     float center, r, z;
     bool last = false;  // beyond x = g
     if (!prism) {
@@ -157,14 +187,13 @@ VOF_HD double alpha64_half(double a, double b, double c, double v) {
     }
     z = fminf(fmaxf(z, -1.f), 1.f);
     const float xf = center + 2.f * r * cosf(acosf(z) * (1.f / 3.f) - 2.09439510239f);
-    double x = (double)xf;
-    if (!(x > 1.0)) x = 1.0;  // also a NaN of a degenerate seed
+    double x = xf > 1.f ? (double)xf : 1.0;  // (1 also for a NaN of a degenerate seed)
     if (lt_pos(hi, x)) x = hi;
     if (lt_pos(p, 1e-20)) return b * x;  // the region is narrower than an ulp
     // Newton: G(x) = p (3x(x - p) + p^2 - 6w) - (x - 1)^3 - (x - g)_+^3
     const float xs = (float)x, t1 = xs - 1.f, t2 = fmaxf(xs - gf, 0.f);
     const double rs = (double)(1.f / (pf * (6.f * xs - 3.f * pf) - 3.f * (t1 * t1 + t2 * t2)));
-    const double k0 = p2 - w6;
+    const double k0 = fma(p, p, -w6);
 #ifdef __CUDACC__
 #pragma unroll
 #endif
@@ -176,6 +205,14 @@ VOF_HD double alpha64_half(double a, double b, double c, double v) {
     if (lt_pos(hi, x)) x = hi;
     return b * x;
 }
+VOF_HD double alpha64_half(double a, double b, double c, double v) {
+    double p, w6, g, x;
+    const int piece = alpha64_piece(a, b, c, v, p, w6, g, x);
+    if (piece == kAlphaCbrt) return alpha64_cbrt(p, w6, b);
+    if (piece == kAlphaSqrt) return alpha64_sqrt(p, w6, b);
+    if (piece == kAlphaCubic) return alpha64_cubic(p, w6, g, b);
+    return x;
+}
 
 // Plane constant of the reflected, sorted normal for a fraction cv in (0, 1).
 VOF_HD double alpha64(double a, double b, double c, double cv) {
@@ -184,20 +221,56 @@ VOF_HD double alpha64(double a, double b, double c, double cv) {
     return flip ? (a + b + c) - x : x;
 }
 
+// A double as a whole number of 2^(eref - 1080), eref >= its biased exponent
+// (bits below that are dropped): |result| < 2^58.
+VOF_HD long long fixed64(double v, int eref) {
+    const long long b = bits64(v);
+    const int e = (int)(b >> 52) & 0x7ff;
+    const long long m = ((b & 0xfffffffffffffLL) | 0x10000000000000LL) << 5;
+    const int sh = eref - e;
+    const long long q = m >> (sh > 62 ? 62 : sh);
+    return b < 0 ? -q : q;
+}
+// A whole number times 2^sh as a double (0 stays 0).
+VOF_HD double scaled64(long long n, int sh) {
+    const double v = (double)n;
+    return n == 0 ? 0.0 : from_bits64(bits64(v) + ((long long)sh << 52));
+}
+VOF_HD unsigned long long mag64(long long v) { return (unsigned long long)(v < 0 ? -v : v); }
+
 // Mixed-Youngs-Centred direction of a stencil (myc_normal in plic.cuh gives
-// the rule), not normalised; returns its L1 norm.  The Youngs sums run
-// through partial sums (51 additions instead of 81); the
-// centred-column candidates, whose own component is +-1, compare by their L1
-// norms instead of three divisions -- the quotients decide only where two
-// norms agree to two ulps, so that symmetric stencils keep their choice.
-VOF_HD double myc_direction64(const double* st, double m[3]) {
-#define VOF_S(i, j, k) st[((k) + 1) * 9 + ((j) + 1) * 3 + ((i) + 1)]
-    // Youngs: differences first (exact between close values), then the
-    // (1, 2, 1) weights along the two other axes
-    auto smooth = [](double lo, double mid, double hi) { return fma(2.0, mid, lo + hi); };
-    double y[3];
+// the rule), not normalised: its largest component lies in 1 .. 2.  The hundred
+// additions run on 64-bit integers (the integer pipes are idle in the FP64
+// kernels): the fractions become whole numbers of 2^-57 of the largest
+// neighbour's binade, 32 times finer than that value's own last place, so that
+// sums and differences are exact and no less accurate than in double.  The
+// candidates compare by T, their L1 norm being 1 + T/2, Youngs against the best
+// candidate in float; near a tie both take the rounded quotients of the rule in
+// double.
+VOF_HD void myc_direction64(const double* st, double m[3]) {
+#define VOF_S(i, j, k) q[((k) + 1) * 9 + ((j) + 1) * 3 + ((i) + 1)]
+    int eref = 600;  // a stencil below 2^-423 counts as empty
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int c = 0; c < 27; ++c) {
+        const int e = (int)(bits64(st[c]) >> 52) & 0x7ff;
+        if (c != 13) eref = e > eref ? e : eref;  // (the centre enters no sum)
+    }
+    if (eref == 0x7ff) {  // an infinity or a NaN beside the cell
+        m[0] = m[1] = m[2] = from_bits64(0x7ff8000000000000LL);
+        return;
+    }
+    long long q[27];
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int c = 0; c < 27; ++c) q[c] = c == 13 ? 0 : fixed64(st[c], eref);
+    // Youngs: differences along the axis, weights (1, 2, 1) along the others
+    auto smooth = [](long long lo, long long mid, long long hi) { return lo + hi + 2 * mid; };
+    long long y[3];
     {
-        double s[3];
+        long long s[3];
 #ifdef __CUDACC__
 #pragma unroll
 #endif
@@ -220,87 +293,111 @@ VOF_HD double myc_direction64(const double* st, double m[3]) {
                               VOF_S(1, j, -1) - VOF_S(1, j, 1));
         y[2] = smooth(s[0], s[1], s[2]);
     }
-    // centred columns: (b, c) components of the candidate along each axis
-    const double cx_b = (((VOF_S(-1, -1, 0) + VOF_S(0, -1, 0)) + VOF_S(1, -1, 0)) -
-                         ((VOF_S(-1, 1, 0) + VOF_S(0, 1, 0)) + VOF_S(1, 1, 0))) * 0.5;
-    const double cx_c = (((VOF_S(-1, 0, -1) + VOF_S(0, 0, -1)) + VOF_S(1, 0, -1)) -
-                         ((VOF_S(-1, 0, 1) + VOF_S(0, 0, 1)) + VOF_S(1, 0, 1))) * 0.5;
-    const double cy_b = (((VOF_S(-1, -1, 0) + VOF_S(-1, 0, 0)) + VOF_S(-1, 1, 0)) -
-                         ((VOF_S(1, -1, 0) + VOF_S(1, 0, 0)) + VOF_S(1, 1, 0))) * 0.5;
-    const double cy_c = (((VOF_S(0, -1, -1) + VOF_S(0, 0, -1)) + VOF_S(0, 1, -1)) -
-                         ((VOF_S(0, -1, 1) + VOF_S(0, 0, 1)) + VOF_S(0, 1, 1))) * 0.5;
-    const double cz_b = (((VOF_S(-1, 0, -1) + VOF_S(-1, 0, 0)) + VOF_S(-1, 0, 1)) -
-                         ((VOF_S(1, 0, -1) + VOF_S(1, 0, 0)) + VOF_S(1, 0, 1))) * 0.5;
-    const double cz_c = (((VOF_S(0, -1, -1) + VOF_S(0, -1, 0)) + VOF_S(0, -1, 1)) -
-                         ((VOF_S(0, 1, -1) + VOF_S(0, 1, 0)) + VOF_S(0, 1, 1))) * 0.5;
+    // centred columns: twice the (b, c) components of the candidate along each axis
+    const long long xb = (VOF_S(-1, -1, 0) + VOF_S(0, -1, 0) + VOF_S(1, -1, 0)) -
+                         (VOF_S(-1, 1, 0) + VOF_S(0, 1, 0) + VOF_S(1, 1, 0));
+    const long long xc = (VOF_S(-1, 0, -1) + VOF_S(0, 0, -1) + VOF_S(1, 0, -1)) -
+                         (VOF_S(-1, 0, 1) + VOF_S(0, 0, 1) + VOF_S(1, 0, 1));
+    const long long yb = (VOF_S(-1, -1, 0) + VOF_S(-1, 0, 0) + VOF_S(-1, 1, 0)) -
+                         (VOF_S(1, -1, 0) + VOF_S(1, 0, 0) + VOF_S(1, 1, 0));
+    const long long yc = (VOF_S(0, -1, -1) + VOF_S(0, 0, -1) + VOF_S(0, 1, -1)) -
+                         (VOF_S(0, -1, 1) + VOF_S(0, 0, 1) + VOF_S(0, 1, 1));
+    const long long zb = (VOF_S(-1, 0, -1) + VOF_S(-1, 0, 0) + VOF_S(-1, 0, 1)) -
+                         (VOF_S(1, 0, -1) + VOF_S(1, 0, 0) + VOF_S(1, 0, 1));
+    const long long zc = (VOF_S(0, -1, -1) + VOF_S(0, -1, 0) + VOF_S(0, -1, 1)) -
+                         (VOF_S(0, 1, -1) + VOF_S(0, 1, 0) + VOF_S(0, 1, 1));
 #undef VOF_S
-    // L1 norms, summed in component order
-    const double lx = (1.0 + abs64(cx_b)) + abs64(cx_c);
-    const double ly = (abs64(cy_b) + 1.0) + abs64(cy_c);
-    const double lz = (abs64(cz_b) + abs64(cz_c)) + 1.0;
-    auto better = [](double l, double best) {  // 1/l > 1/best as rounded quotients
-        const long long dl = bits64(best) - bits64(l);
-        if (dl > 2) return true;
-        if (dl <= 0) return false;
-        return 1.0 / l > 1.0 / best;
+    // T of each candidate, compared in units of 2^-52; near a tie by the
+    // rounded quotients of the rule (ties to the lower axis)
+    const int sh = eref - 1081;  // half of one unit is 2^sh
+    const int k52 = 1028 - eref, kq = k52 > 63 ? 63 : (k52 < 0 ? 0 : k52);
+    const unsigned long long tx = mag64(xb) + mag64(xc), ty = mag64(yb) + mag64(yc), tz = mag64(zb) + mag64(zc);
+    auto l1_of = [&](int axis) {  // the norm with every sum rounded in the rule's order
+        const int sa = axis == 0 ? 1 : (axis == 1 ? 3 : 9), sb = axis == 0 ? 3 : 1, sc = axis == 2 ? 3 : 9;
+        auto column = [&](int o) { return (st[13 + o - sa] + st[13 + o]) + st[13 + o + sa]; };
+        const double b = abs64((column(-sb) - column(sb)) * 0.5), c = abs64((column(-sc) - column(sc)) * 0.5);
+        return axis == 0 ? (1.0 + b) + c : (axis == 1 ? (b + 1.0) + c : (b + c) + 1.0);
     };
-    double lbest = lx;
-    m[0] = negative64(y[0]) ? -1.0 : 1.0;
-    m[1] = cx_b;
-    m[2] = cx_c;
-    if (better(ly, lbest)) {
-        lbest = ly;
-        m[0] = cy_b;
-        m[1] = negative64(y[1]) ? -1.0 : 1.0;
-        m[2] = cy_c;
-    }
-    if (better(lz, lbest)) {
-        lbest = lz;
-        m[0] = cz_b;
-        m[1] = cz_c;
-        m[2] = negative64(y[2]) ? -1.0 : 1.0;
-    }
-    const double ax = abs64(y[0]), ay = abs64(y[1]), az = abs64(y[2]);
-    const double ny = ax + ay + az;
-    double ymax = lt_pos(ax, ay) ? ay : ax;
-    ymax = lt_pos(ymax, az) ? az : ymax;
-    // Youngs where ymax / ny < 1 / lbest (the quotients near a tie)
+    auto better = [&](unsigned long long t_new, int a_new, unsigned long long t_best, int a_best) {
+        const long long d = (long long)(t_best >> kq) - (long long)(t_new >> kq);
+        if (d > 4) return true;
+        if (d < -4) return false;
+        const double l_new = l1_of(a_new), l_best = l1_of(a_best);
+        const long long u = bits64(l_best) - bits64(l_new);  // (a quotient falls as its norm rises)
+        return u > 2 || (u > 0 && 1.0 / l_new > 1.0 / l_best);
+    };
+    int axis = 0;
+    unsigned long long t = tx;
+    if (better(ty, 1, t, axis)) { axis = 1; t = ty; }
+    if (better(tz, 2, t, axis)) { axis = 2; t = tz; }
+    // Youngs where ymax / ny < 1 / (1 + T/2): ymax T/2 < ny - ymax
+    const unsigned long long ax = mag64(y[0]), ay = mag64(y[1]), az = mag64(y[2]);
+    unsigned long long ymax = ax > ay ? ax : ay;
+    ymax = ymax > az ? ymax : az;
+    const unsigned long long rest = ax + ay + az - ymax;
     bool youngs = false;
-    if (le_pos(1e-30, ny)) {
-        const double t = ymax * lbest;
-        const long long dl = bits64(ny) - bits64(t);
-        youngs = dl > 4 || (dl >= -4 && ymax / ny < 1.0 / lbest);
+    // (the rule's ny >= 1e-30: one unit, 2^(eref - 1080), reaches it from eref = 981)
+    const double ny = (double)(ax + ay + az);  // below 2^63.6
+    if (ymax != 0 && (eref >= 981 || le_pos(1e-30, from_bits64(bits64(ny) + ((long long)(eref - 1080) << 52))))) {
+#ifdef __CUDA_ARCH__
+        const float half_t = __ull2float_rn(t) * __int_as_float((sh + 127 < 1 ? 0 : sh + 127) << 23);
+        const float lf = __ull2float_rn(ymax) * half_t, rf = __ull2float_rn(rest);
+#else
+        const float half_t = sh + 127 < 1 ? 0.f : ldexpf((float)t, sh);
+        const float lf = (float)ymax * half_t, rf = (float)rest;
+#endif
+        youngs = lf < rf;
+        if (fabsf(lf - rf) <= 1e-5f * (lf + rf)) youngs = (double)ymax * scaled64((long long)t, sh) < (double)rest;
     }
-    if (youngs) {
-        m[0] = y[0];
-        m[1] = y[1];
-        m[2] = y[2];
-        return ny;
+    if (youngs) {  // the largest component to 1 .. 2
+#ifdef __CUDA_ARCH__
+        const int top = __clzll((long long)ymax) - 63;
+#else
+        const int top = __builtin_clzll(ymax) - 63;
+#endif
+        m[0] = scaled64(y[0], top);
+        m[1] = scaled64(y[1], top);
+        m[2] = scaled64(y[2], top);
+        return;
     }
-    return lbest;
+    const long long db = axis == 0 ? xb : (axis == 1 ? yb : zb), dc = axis == 0 ? xc : (axis == 1 ? yc : zc);
+    const double own = (axis == 0 ? y[0] : (axis == 1 ? y[1] : y[2])) < 0 ? -1.0 : 1.0;
+    const double mb = scaled64(db, sh), mc = scaled64(dc, sh);
+    m[0] = axis == 0 ? own : mb;
+    m[1] = axis == 1 ? own : (axis == 0 ? mb : mc);
+    m[2] = axis == 2 ? own : mc;
 }
 
-// Flux through a face of the donor of fraction cv in (0, 1) with normal
-// direction m (any scale); s is the signed Courant number.  In the frame
-// reflected to non-negative components the swept slab [1 - s, 1] (s > 0) or
-// [0, |s|] (s < 0) keeps or swaps its end with the sign of m_d; it is mapped
-// onto the unit cube by n_d -> n_d |s|, alpha -> alpha - n_d x0.
-VOF_HD double face_flux64(const double m[3], double cv, int d, double s) {
-    double n0 = abs64(m[0]), n1 = abs64(m[1]), n2 = abs64(m[2]);
-    double a = n0, b = n1, c = n2;
-    sort3_pos(a, b, c);
-    const double al = alpha64(a, b, c, cv);
+// The swept slab of a face flux mapped onto the unit cube.  In the frame
+// reflected to non-negative components n the slab [1 - s, 1] (s > 0) or
+// [0, |s|] (s < 0) keeps or swaps its end with the sign of m_d; then n_d ->
+// n_d |s|, alpha -> alpha - n_d x0.  n: sorted on return; returns the constant.
+VOF_HD double slab64(const double m[3], double al, int d, double s, double n[3]) {
+    n[0] = abs64(m[0]);
+    n[1] = abs64(m[1]);
+    n[2] = abs64(m[2]);
     const double as = abs64(s);
-    const double nd = d == 0 ? n0 : (d == 1 ? n1 : n2), md = d == 0 ? m[0] : (d == 1 ? m[1] : m[2]);
+    const double nd = d == 0 ? n[0] : (d == 1 ? n[1] : n[2]), md = d == 0 ? m[0] : (d == 1 ? m[1] : m[2]);
     const bool far_end = negative64(s) == negative64(md);
     const double x = far_end ? fma(-nd, 1.0 - as, al) : al;
     const double sd = nd * as;
-    if (d == 0) n0 = sd;
-    else if (d == 1) n1 = sd;
-    else n2 = sd;
-    sort3_pos(n0, n1, n2);
-    if (!lt_pos(0.0, n2)) return bits64(x) > 0 ? s : 0.0;
-    return s * vol64(n0, n1, n2, x);
+    if (d == 0) n[0] = sd;
+    else if (d == 1) n[1] = sd;
+    else n[2] = sd;
+    sort3_pos(n[0], n[1], n[2]);
+    return x;
+}
+
+// Flux through a face of the donor of fraction cv in (0, 1) with normal
+// direction m (largest component within 2^-20 .. 2^20); s is the signed
+// Courant number.
+VOF_HD double face_flux64(const double m[3], double cv, int d, double s) {
+    double a = abs64(m[0]), b = abs64(m[1]), c = abs64(m[2]);
+    sort3_pos(a, b, c);
+    double n[3];
+    const double x = slab64(m, alpha64(a, b, c, cv), d, s, n);
+    if (!lt_pos(0.0, n[2])) return bits64(x) > 0 ? s : 0.0;
+    return s * vol64(n[0], n[1], n[2], x);
 }
 
 }  // namespace vof

@@ -56,3 +56,43 @@ def test_plane_constant_and_volume(vof, n, scale):
     vo = np.array([O.plic_volume(m[t], al[t]) for t in range(len(c))])
     assert np.abs(vo - c).max() <= 1e-14
 
+
+
+def pattern(kind, rng, shape=(7, 9, 11)):
+    k, j, i = np.meshgrid(*[np.arange(s) for s in shape], indexing="ij")
+    if kind == "diagonal":  # equal quotients of two or three axes
+        c = np.clip((i + j + k - 13) * 0.25 + 0.5, 0.0, 1.0)
+    elif kind == "axis":
+        c = np.clip((k - 3) * 0.75 + 0.5, 0.0, 1.0)
+    elif kind == "sixteenths":
+        c = rng.integers(0, 17, shape) / 16.0
+    elif kind == "mixed":
+        c = np.where(rng.random(shape) < 0.3, 0.0, np.where(rng.random(shape) < 0.5, 1.0, rng.random(shape)))
+    elif kind == "flat":  # differences far below the values
+        c = 0.5 + 1e-6 * rng.standard_normal(shape)
+    elif kind == "spread":  # sixteen decades
+        c = 10.0 ** (-16.0 * rng.random(shape))
+    else:  # residues about the least norm at which the rule takes Youngs' normal
+        c = 10.0 ** (-29.0 - 3.0 * rng.random(shape))
+    return np.ascontiguousarray(c, dtype=np.float64)
+
+
+# Tolerance: a sum of the rule has at most nine terms of weight up to 2 and
+# 16 values' weight in all, so its rounding is below 8 * 16 * 2^-53 = 1.5e-14
+# of the largest value; a component of the normal is off by that over the
+# largest component (0.3 or more of the values in all but the flat field, whose
+# differences are 1e-6 of them).  A centred-column normal has a component 1.
+@pytest.mark.parametrize("kind, tol", [("diagonal", 1e-13), ("axis", 1e-13), ("sixteenths", 1e-13),
+                                       ("mixed", 1e-13), ("flat", 1e-7), ("spread", 1e-13),
+                                       ("residue", 1e-13)])
+def test_normal_direction(vof, kind, tol):
+    c = pattern(kind, np.random.default_rng(5))
+    cfg = vof.make_config(c.shape[2], c.shape[1], c.shape[0])
+    f = torch.from_numpy(c[None]).to(DEV)
+    u = torch.zeros((3,) + c.shape, dtype=torch.float64, device=DEV)
+    ctx = vof.Context(cfg, f, u)
+    m = ctx.vof_normals(0).cpu().numpy()
+    ctx.close()
+    o = O.normals(c)
+    assert np.isfinite(m).all()
+    assert np.abs(m - o).max() <= tol

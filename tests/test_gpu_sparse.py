@@ -103,3 +103,21 @@ def test_recolour_after_replaced_fields(vof):
         ctx.close()
     assert out[0][1] == out[1][1] and out[0][1] > 0
     assert np.array_equal(out[0][0], out[1][0])
+
+
+@pytest.mark.parametrize("band", [0.0, 1e-3, 0.4999])
+@pytest.mark.parametrize("shape,K", [((3, 4, 5), 1), ((9, 8, 64), 3)])
+def test_refined_faces(vof, shape, K, band):
+    """The faces queued for the FP64 step of the mixed path: none, a few, nearly
+    all, with less than one block of faces and with a part-filled last block."""
+    u = synth.solenoidal_velocity(shape, 4, 0.5, 0.6, 3)
+    dt = synth.dt_for_cfl(u, 0.4)
+    c_d = torch.from_numpy(field_set(shape, K, 2)).to(DEV, torch.float32).contiguous()
+    u_d = torch.from_numpy(u).to(DEV, torch.float32).contiguous()
+    want, _ = O.advect(c_d.cpu().numpy().astype(np.float64), u_d.cpu().numpy().astype(np.float64), dt, 1.0, 1)
+    cfg = vof.make_config(shape[2], shape[1], shape[0], k_capacity=K, k_active=K, precision=1, recolour=0,
+                          alpha_fp64_band=band)
+    ctx = vof.Context(cfg, c_d, u_d)
+    ctx.vof_step(dt, 1)
+    assert np.abs(c_d.cpu().numpy() - want).max() <= 1e-5
+    ctx.close()
