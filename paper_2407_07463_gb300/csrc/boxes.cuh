@@ -577,10 +577,14 @@ __global__ void __launch_bounds__(256) k_list_patch(const __grid_constant__ BoxS
 // set to zero.
 //
 // In double the kernel is bound by FP64 issue (1/64 of the FP32 rate), so
-// its time is its count of FP64 instructions: the forms of plic64.cuh took
-// it from 6.2 to 1.08 ms per sweep of the 256^3, K = 8, phi = 0.3 box (2.7 M
-// faces), and a sweep of 32^3 with 8 drops, where one warp's chain is the
-// time, from 78 to 22 us with its other launches.
+// its time is its count of FP64 warp instructions: the forms of plic64.cuh, and
+// the roots taken by piece (cubic, square root, cube root: the block's faces are
+// reordered so that a warp runs one piece, at most two, instead of all three
+// with nine lanes each), took it from 6.2 to 0.72 ms per sweep of the 256^3,
+// K = 8, phi = 0.3 box (2.7 M faces; 1.08 ms before the reordering and before
+// the volume's pieces became selects: 212 -> 88 to 120 FP64 instructions per
+// warp of faces), and a sweep of 32^3 with 8 drops, where one warp's chain is
+// the time, from 78 to 20 us with its other launches.
 //
 // In FP32 the faces whose fraction lies within `band` of 0 or 1 (one in six)
 // take an FP64 step: they are compacted to the first threads of the block, so
@@ -594,7 +598,7 @@ __global__ void __launch_bounds__(kFaceTile) k_face_flux_bx(const __grid_constan
                                                             int* __restrict__ next_count) {
     constexpr bool kBanded = std::is_same<T, float>::value;
     constexpr int kWarps = kFaceTile / 32;
-    __shared__ T s_q[kBanded ? 4 : 1][kBanded ? kFaceTile : 1];  // queued normals and fractions, then constants
+    __shared__ T s_q[4][kFaceTile];  // queued normals and fractions (a piece's variables), then constants
     __shared__ int s_n[kWarps];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     if (blockIdx.x == 0 && t == 0) *next_count = 0;
@@ -611,12 +615,8 @@ __global__ void __launch_bounds__(kFaceTile) k_face_flux_bx(const __grid_constan
             T st[27];
             gather_stencil_ijk(sweep_in(B, sweep) + (size_t)fc.f * B.g.N, fc.di, fc.dj, fc.dk, B.g, st);
             cv = st[13];
-            if constexpr (kBanded) {
-                myc_normal(st, m);
-            } else {
-                myc_direction64(st, m);
-                *dst = face_flux64(m, cv, d, sv);
-            }
+            if constexpr (kBanded) myc_normal(st, m);
+            else myc_direction64(st, m);
         }
         if constexpr (kBanded) {
             const bool queue = valid && (cv < band || cv > T(1) - band);
@@ -643,6 +643,37 @@ __global__ void __launch_bounds__(kFaceTile) k_face_flux_bx(const __grid_constan
             if (queue) alpha = s_q[3][at];
             if (valid) *dst = face_flux(m, alpha, d, sv);
             // (s_q is written again only after the next tile's first barrier)
+        } else {
+            // the roots by piece: the faces of a piece on neighbouring threads
+            T a = abs64(m[0]), b = abs64(m[1]), c = abs64(m[2]);
+            sort3_pos(a, b, c);
+            const bool flip = lt_pos(T(0.5), cv);
+            T p, w6, g, x;
+            const int piece = valid ? alpha64_piece(a, b, c, flip ? T(1) - cv : cv, p, w6, g, x) : kAlphaLinear;
+            const unsigned v0 = __ballot_sync(0xffffffffu, piece == 0), v1 = __ballot_sync(0xffffffffu, piece == 1),
+                           v2 = __ballot_sync(0xffffffffu, piece == 2);
+            if (lane == 0) s_n[warp] = __popc(v0) | __popc(v1) << 8 | __popc(v2) << 16;
+            __syncthreads();
+            int before = 0, all = 0;  // three counts of up to 128, 8 bits each
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) {
+                before += w < warp ? s_n[w] : 0;
+                all += s_n[w];
+            }
+            const int n0 = all & 255, n1 = n0 + (all >> 8 & 255), n2 = n1 + (all >> 16);
+            const unsigned mine = piece == 0 ? v0 : (piece == 1 ? v1 : v2);
+            const int at = (piece == 0 ? 0 : (piece == 1 ? n0 : n1)) + (before >> (8 * piece) & 255) +
+                           __popc(mine & ((1u << lane) - 1u));
+            if (piece != kAlphaLinear) {
+                s_q[0][at] = p;
+                s_q[1][at] = w6;
+                s_q[2][at] = g;
+            }
+            __syncthreads();
+            if (t < n2) s_q[3][t] = alpha64_root(t < n0 ? 0 : (t < n1 ? 1 : 2), s_q[0][t], s_q[1][t], s_q[2][t]);
+            __syncthreads();
+            if (piece != kAlphaLinear) x = b * s_q[3][at];
+            if (valid) *dst = face_flux64_at(m, flip ? (a + b + c) - x : x, d, sv);
         }
     }
 }

@@ -19,8 +19,8 @@
 // without contraction give the same bits.
 //
 // Against quadruple precision on a million random planes, fractions and
-// Courant numbers (tiny and zero components included): flux within 4.6e-16
-// (mean 1.17e-17), plane constant within 3.1e-16 (mean 3.4e-17); the
+// Courant numbers (tiny and zero components included): flux within 3.5e-16
+// (mean 1.18e-17), plane constant within 3.1e-16 (mean 3.4e-17); the
 // piecewise Gauss evaluation and its Newton inversion that stood here before
 // gave 5.6e-16 (1.37e-17) and 3.6e-16 (4.2e-17).  Times: k_face_flux_bx.
 #pragma once
@@ -62,6 +62,31 @@ VOF_HD bool le_pos(double p, double q) { return bits64(p) <= bits64(q); }
 // max(v, 0) for any v (-0 gives +0).
 VOF_HD double plus64(double v) { return bits64(v) < 0 ? 0.0 : v; }
 
+// Conversions on the integer ALU (the FP64 unit does them otherwise).  The
+// float of v >= 0, cut off instead of rounded: 0 below FP32's normal range, v
+// below 2^127.
+VOF_HD float low_float(double v) {
+    const long long b = bits64(v) - (896LL << 52);
+    const int f = b < (1LL << 52) ? 0 : (int)(b >> 29);
+#ifdef __CUDA_ARCH__
+    return __int_as_float(f);
+#else
+    float r;
+    __builtin_memcpy(&r, &f, 4);
+    return r;
+#endif
+}
+// The double of a float that is positive and normal.
+VOF_HD double wide(float v) {
+#ifdef __CUDA_ARCH__
+    const int f = __float_as_int(v);
+#else
+    int f;
+    __builtin_memcpy(&f, &v, 4);
+#endif
+    return from_bits64(((long long)f << 29) + (896LL << 52));
+}
+
 VOF_HD void sort3_pos(double& a, double& b, double& c) {
     double t;
     if (lt_pos(b, a)) { t = a; a = b; b = t; }
@@ -76,53 +101,43 @@ VOF_HD double cbrt64(double t) {
     const int e = (int)(bits64(t) >> 52) - 1023;          // >= -997
     const int k = (e + 1200) / 3 - 400;                   // floor(e / 3)
     const double m = t * from_bits64((long long)(1023 - 3 * k) << 52);  // in [1, 8)
-    const float yf = cbrtf((float)m);
-    const double r = (double)(1.f / (3.f * yf * yf));
-    double y = (double)yf;
+    const float yf = cbrtf(low_float(m));
+    const double r = wide(1.f / (3.f * yf * yf));
+    double y = wide(yf);
     y = fma(-fma(y * y, y, -m), r, y);
     y = fma(-fma(y * y, y, -m), r, y);
     return y * from_bits64((long long)(1023 + k) << 52);
 }
 
 // Volume under the plane a x + b y + c z < x in the unit cube, sorted
-// 0 <= a <= b <= c, c > 0, 0 <= x <= (a + b + c) / 2, by its piece.
-enum VolPiece { kVolTip = 0, kVolPrism = 1, kVolEdge = 2, kVolCorner = 3 };
-VOF_HD int vol64_piece(double a, double b, double c, double x) {
-    if (le_pos(x, a)) return kVolTip;
-    if (lt_pos(a + b, x)) return kVolPrism;  // (x <= S/2 leaves it to c > a + b)
-    return le_pos(x, b) ? kVolEdge : kVolCorner;
-}
-VOF_HD double vol64_of(int piece, double a, double b, double c, double x) {
-    double num, den;
-    if (piece == kVolTip) {
-        num = x * x * x;
-        den = 6.0 * a * b * c;
-    } else if (piece == kVolPrism) {
-        num = fma(2.0, x, -(a + b));
-        den = 2.0 * c;
-    } else {
-        num = fma(3.0 * x, x - a, a * a);
-        den = 6.0 * b * c;
-        if (piece == kVolCorner) {
-            const double tb = x - b, tc = plus64(x - c);
-            num = fma(a, num, -fma(tb * tb, tb, tc * tc * tc));
-            den *= a;
-        }
-    }
+// 0 <= a <= b <= c, c > 0, 0 <= x <= (a + b + c) / 2: numerator and divisor of
+// every piece, taken by selects (19 products and sums; as branches the lanes of
+// a warp paid for 24 and the branches).
+VOF_HD double vol64_half(double a, double b, double c, double x) {
+    const double ab = a + b, e = 6.0 * b * c, ea = e * a;
+    const double tb = x - b, tc = plus64(x - c);
+    const double q = fma(3.0 * x, x - a, a * a);
+    const bool tip = le_pos(x, a);
+    const bool prism = lt_pos(ab, x);          // (x <= S/2 leaves it to c > a + b)
+    const bool corner = lt_pos(b, x);          // not at x = b, where a may be zero
+    double num = corner ? fma(a, q, -fma(tb * tb, tb, tc * tc * tc)) : q;
+    double den = corner ? ea : e;
+    num = prism ? fma(2.0, x, -ab) : num;
+    den = prism ? 2.0 * c : den;
+    num = tip ? x * x * x : num;
+    den = tip ? ea : den;
     // a divisor this small belongs to a plane whose volume is below 1e-90
     return lt_pos(den, 1e-290) ? 0.0 : num / den;
-}
-VOF_HD double vol64_half(double a, double b, double c, double x) {
-    return vol64_of(vol64_piece(a, b, c, x), a, b, c, x);
 }
 
 // The same for any x; S = a + b + c > 0.
 VOF_HD double vol64(double a, double b, double c, double x) {
-    const double S = a + b + c, y = S - x;
     if (bits64(x) <= 0) return 0.0;
+    const double S = a + b + c, y = S - x;
     if (bits64(y) <= 0) return 1.0;
-    if (lt_pos(y, x)) return 1.0 - vol64_half(a, b, c, y);
-    return vol64_half(a, b, c, x);
+    const bool flip = lt_pos(y, x);  // (one copy of the pieces for both halves)
+    const double v = vol64_half(a, b, c, flip ? y : x);
+    return flip ? 1.0 - v : v;
 }
 
 // Root x in (0, S/2] of vol64_half(a, b, c, x) = v, 0 < v <= 1/2, sorted
@@ -132,22 +147,24 @@ VOF_HD double vol64(double a, double b, double c, double x) {
 //   c >= a + b, 2w >= 1 + p:  the prism, x = w + (1 + p)/2
 //   else  p (3x(x - p) + p^2 - 6w) = (x - 1)^3 + (x - g)_+^3, seeded by the
 //   middle root of the cubic in trigonometric form (alpha_sorted_pw).
-enum AlphaPiece { kAlphaLinear = 0, kAlphaCbrt = 1, kAlphaSqrt = 2, kAlphaCubic = 3 };
+enum AlphaPiece { kAlphaCubic = 0, kAlphaSqrt = 1, kAlphaCbrt = 2, kAlphaLinear = 3 };
 // 1 / b for b within FP32's range: two Newton steps from the FP32 quotient.
 VOF_HD double rcp64(double b) {
-    double r = (double)(1.f / (float)b);
+    double r = wide(1.f / low_float(b));
     r = fma(fma(-b, r, 1.0), r, r);
     return fma(fma(-b, r, 1.0), r, r);
 }
-// The piece the root lies in and its scaled variables p, w6 = 6w and g (g only
-// for the cubic); the linear pieces' root in x.  c within 2^-20 .. 2^20.
+// The piece the root lies in with its variables p, w6 = 6w and g; root / b is
+// alpha64_root of these, the linear pieces' root is x.  c within 2^-20 .. 2^20.
 VOF_HD int alpha64_piece(double a, double b, double c, double v, double& p, double& w6, double& g, double& x) {
     const double cv = c * v;
     x = cv;
+    p = w6 = g = 0.0;
     if (lt_pos(b, 1e-30 * c)) return kAlphaLinear;  // a plane across one axis (off by < 1e-30 c)
     const double ib = rcp64(b);
     p = a * ib;
     w6 = 6.0 * cv * ib;
+    g = c * ib;
     const double p2 = p * p;
     if (le_pos(w6, p2)) return kAlphaCbrt;
     if (!negative64(fma(3.0, 1.0 - p, p2) - w6)) return kAlphaSqrt;
@@ -156,16 +173,11 @@ VOF_HD int alpha64_piece(double a, double b, double c, double v, double& p, doub
         x = fma(0.5, ab, cv);
         return kAlphaLinear;
     }
-    g = c * ib;
     return kAlphaCubic;
 }
-VOF_HD double alpha64_cbrt(double p, double w6, double b) { return b * cbrt64(p * w6); }
-VOF_HD double alpha64_sqrt(double p, double w6, double b) {
-    return b * (0.5 * (p + sqrt(fma(-1.0 / 3.0, p * p, (4.0 / 3.0) * w6))));
-}
-VOF_HD double alpha64_cubic(double p, double w6, double g, double b) {
+VOF_HD double alpha64_cubic(double p, double w6, double g) {
     // seed
-    const float pf = (float)p, gf = (float)g, wf = (float)w6 * (1.f / 6.f);
+    const float pf = low_float(p), gf = low_float(g), wf = low_float(w6) * (1.f / 6.f);
     const double p1 = 1.0 + p;
     const bool prism = le_pos(p1, g);
     const double hi = prism ? p1 : 0.5 * (p1 + g);
@@ -187,11 +199,11 @@ VOF_HD double alpha64_cubic(double p, double w6, double g, double b) {
     }
     z = fminf(fmaxf(z, -1.f), 1.f);
     const float xf = center + 2.f * r * cosf(acosf(z) * (1.f / 3.f) - 2.09439510239f);
-    double x = xf > 1.f ? (double)xf : 1.0;  // (1 also for a NaN of a degenerate seed)
+    double x = xf > 1.f ? wide(xf) : 1.0;  // (1 also for a NaN of a degenerate seed)
     if (lt_pos(hi, x)) x = hi;
-    if (lt_pos(p, 1e-20)) return b * x;  // the region is narrower than an ulp
+    if (lt_pos(p, 1e-20)) return x;  // the region is narrower than an ulp
     // Newton: G(x) = p (3x(x - p) + p^2 - 6w) - (x - 1)^3 - (x - g)_+^3
-    const float xs = (float)x, t1 = xs - 1.f, t2 = fmaxf(xs - gf, 0.f);
+    const float xs = low_float(x), t1 = xs - 1.f, t2 = fmaxf(xs - gf, 0.f);
     const double rs = (double)(1.f / (pf * (6.f * xs - 3.f * pf) - 3.f * (t1 * t1 + t2 * t2)));
     const double k0 = fma(p, p, -w6);
 #ifdef __CUDACC__
@@ -202,16 +214,17 @@ VOF_HD double alpha64_cubic(double p, double w6, double g, double b) {
         const double G = fma(p, fma(3.0 * x, x - p, k0), -fma(tb * tb, tb, tc * tc * tc));
         x = fma(-G, rs, x);
     }
-    if (lt_pos(hi, x)) x = hi;
-    return b * x;
+    return lt_pos(hi, x) ? hi : x;
+}
+VOF_HD double alpha64_root(int piece, double p, double w6, double g) {
+    if (piece == kAlphaCubic) return alpha64_cubic(p, w6, g);
+    if (piece == kAlphaSqrt) return 0.5 * (p + sqrt(fma(-1.0 / 3.0, p * p, (4.0 / 3.0) * w6)));
+    return cbrt64(p * w6);
 }
 VOF_HD double alpha64_half(double a, double b, double c, double v) {
     double p, w6, g, x;
     const int piece = alpha64_piece(a, b, c, v, p, w6, g, x);
-    if (piece == kAlphaCbrt) return alpha64_cbrt(p, w6, b);
-    if (piece == kAlphaSqrt) return alpha64_sqrt(p, w6, b);
-    if (piece == kAlphaCubic) return alpha64_cubic(p, w6, g, b);
-    return x;
+    return piece == kAlphaLinear ? x : b * alpha64_root(piece, p, w6, g);
 }
 
 // Plane constant of the reflected, sorted normal for a fraction cv in (0, 1).
@@ -231,12 +244,24 @@ VOF_HD long long fixed64(double v, int eref) {
     const long long q = m >> (sh > 62 ? 62 : sh);
     return b < 0 ? -q : q;
 }
-// A whole number times 2^sh as a double (0 stays 0).
-VOF_HD double scaled64(long long n, int sh) {
-    const double v = (double)n;
-    return n == 0 ? 0.0 : from_bits64(bits64(v) + ((long long)sh << 52));
-}
 VOF_HD unsigned long long mag64(long long v) { return (unsigned long long)(v < 0 ? -v : v); }
+VOF_HD int clz64(unsigned long long v) {
+#ifdef __CUDA_ARCH__
+    return __clzll((long long)v);
+#else
+    return __builtin_clzll(v);
+#endif
+}
+// A whole number times 2^sh as a double, rounded to 53 bits (0 stays 0).
+VOF_HD double scaled64(long long n, int sh) {
+    const unsigned long long u = mag64(n);
+    if (u == 0) return 0.0;
+    const int lz = clz64(u);
+    const unsigned long long top = u << lz;
+    const long long r = (long long)((top >> 11) + ((top >> 10) & 1));  // 2^52 .. 2^53
+    const long long b = r + ((long long)(1085 - lz + sh) << 52);
+    return from_bits64(n < 0 ? b | (long long)0x8000000000000000ULL : b);
+}
 
 // Mixed-Youngs-Centred direction of a stencil (myc_normal in plic.cuh gives
 // the rule), not normalised: its largest component lies in 1 .. 2.  The hundred
@@ -307,8 +332,8 @@ VOF_HD void myc_direction64(const double* st, double m[3]) {
     const long long zc = (VOF_S(0, -1, -1) + VOF_S(0, -1, 0) + VOF_S(0, -1, 1)) -
                          (VOF_S(0, 1, -1) + VOF_S(0, 1, 0) + VOF_S(0, 1, 1));
 #undef VOF_S
-    // T of each candidate, compared in units of 2^-52; near a tie by the
-    // rounded quotients of the rule (ties to the lower axis)
+    // T of each candidate, compared in units of 2^-52; those near the least by
+    // the rounded quotients of the rule (ties to the lower axis)
     const int sh = eref - 1081;  // half of one unit is 2^sh
     const int k52 = 1028 - eref, kq = k52 > 63 ? 63 : (k52 < 0 ? 0 : k52);
     const unsigned long long tx = mag64(xb) + mag64(xc), ty = mag64(yb) + mag64(yc), tz = mag64(zb) + mag64(zc);
@@ -318,27 +343,35 @@ VOF_HD void myc_direction64(const double* st, double m[3]) {
         const double b = abs64((column(-sb) - column(sb)) * 0.5), c = abs64((column(-sc) - column(sc)) * 0.5);
         return axis == 0 ? (1.0 + b) + c : (axis == 1 ? (b + 1.0) + c : (b + c) + 1.0);
     };
-    auto better = [&](unsigned long long t_new, int a_new, unsigned long long t_best, int a_best) {
-        const long long d = (long long)(t_best >> kq) - (long long)(t_new >> kq);
-        if (d > 4) return true;
-        if (d < -4) return false;
-        const double l_new = l1_of(a_new), l_best = l1_of(a_best);
-        const long long u = bits64(l_best) - bits64(l_new);  // (a quotient falls as its norm rises)
-        return u > 2 || (u > 0 && 1.0 / l_new > 1.0 / l_best);
-    };
-    int axis = 0;
-    unsigned long long t = tx;
-    if (better(ty, 1, t, axis)) { axis = 1; t = ty; }
-    if (better(tz, 2, t, axis)) { axis = 2; t = tz; }
+    unsigned long long t = tx < ty ? tx : ty;
+    t = t < tz ? t : tz;
+    const unsigned long long near_t = (t >> kq) + 4;
+    const bool nx = (tx >> kq) <= near_t, ny = (ty >> kq) <= near_t, nz = (tz >> kq) <= near_t;
+    int axis = nx ? 0 : (ny ? 1 : 2);
+    if ((nx && (ny || nz)) || (ny && nz)) {
+        double best = l1_of(axis);
+#ifdef __CUDACC__
+#pragma unroll 1
+#endif
+        for (int other = axis + 1; other < 3; ++other) {
+            if (other == 1 ? !ny : !nz) continue;
+            const double l = l1_of(other);
+            const long long u = bits64(best) - bits64(l);  // (a quotient falls as its norm rises)
+            if (u > 2 || (u > 0 && 1.0 / l > 1.0 / best)) {
+                best = l;
+                axis = other;
+            }
+        }
+        t = axis == 0 ? tx : (axis == 1 ? ty : tz);
+    }
     // Youngs where ymax / ny < 1 / (1 + T/2): ymax T/2 < ny - ymax
     const unsigned long long ax = mag64(y[0]), ay = mag64(y[1]), az = mag64(y[2]);
     unsigned long long ymax = ax > ay ? ax : ay;
     ymax = ymax > az ? ymax : az;
     const unsigned long long rest = ax + ay + az - ymax;
     bool youngs = false;
-    // (the rule's ny >= 1e-30: one unit, 2^(eref - 1080), reaches it from eref = 981)
-    const double ny = (double)(ax + ay + az);  // below 2^63.6
-    if (ymax != 0 && (eref >= 981 || le_pos(1e-30, from_bits64(bits64(ny) + ((long long)(eref - 1080) << 52))))) {
+    // (the rule's |y|_1 >= 1e-30: one unit, 2^(eref - 1080), reaches it from eref = 981)
+    if (ymax != 0 && (eref >= 981 || le_pos(1e-30, scaled64((long long)((ymax + rest) >> 2), eref - 1078)))) {
 #ifdef __CUDA_ARCH__
         const float half_t = __ull2float_rn(t) * __int_as_float((sh + 127 < 1 ? 0 : sh + 127) << 23);
         const float lf = __ull2float_rn(ymax) * half_t, rf = __ull2float_rn(rest);
@@ -347,25 +380,23 @@ VOF_HD void myc_direction64(const double* st, double m[3]) {
         const float lf = (float)ymax * half_t, rf = (float)rest;
 #endif
         youngs = lf < rf;
-        if (fabsf(lf - rf) <= 1e-5f * (lf + rf)) youngs = (double)ymax * scaled64((long long)t, sh) < (double)rest;
+        if (fabsf(lf - rf) <= 1e-5f * (lf + rf))
+            youngs = scaled64((long long)ymax, 0) * scaled64((long long)t, sh) < scaled64((long long)(rest >> 1), 1);
     }
-    if (youngs) {  // the largest component to 1 .. 2
-#ifdef __CUDA_ARCH__
-        const int top = __clzll((long long)ymax) - 63;
-#else
-        const int top = __builtin_clzll(ymax) - 63;
-#endif
-        m[0] = scaled64(y[0], top);
-        m[1] = scaled64(y[1], top);
-        m[2] = scaled64(y[2], top);
+    // Youngs' largest component goes to 1 .. 2
+    const long long cb = axis == 0 ? xb : (axis == 1 ? yb : zb), cc = axis == 0 ? xc : (axis == 1 ? yc : zc);
+    const int ms = youngs ? clz64(ymax) - 63 : sh;
+    const double m0 = scaled64(youngs ? y[0] : cb, ms), m1 = scaled64(youngs ? y[1] : cc, ms);
+    if (youngs) {
+        m[0] = m0;
+        m[1] = m1;
+        m[2] = scaled64(y[2], ms);
         return;
     }
-    const long long db = axis == 0 ? xb : (axis == 1 ? yb : zb), dc = axis == 0 ? xc : (axis == 1 ? yc : zc);
     const double own = (axis == 0 ? y[0] : (axis == 1 ? y[1] : y[2])) < 0 ? -1.0 : 1.0;
-    const double mb = scaled64(db, sh), mc = scaled64(dc, sh);
-    m[0] = axis == 0 ? own : mb;
-    m[1] = axis == 1 ? own : (axis == 0 ? mb : mc);
-    m[2] = axis == 2 ? own : mc;
+    m[0] = axis == 0 ? own : m0;
+    m[1] = axis == 1 ? own : (axis == 0 ? m0 : m1);
+    m[2] = axis == 2 ? own : m1;
 }
 
 // The swept slab of a face flux mapped onto the unit cube.  In the frame
@@ -388,16 +419,20 @@ VOF_HD double slab64(const double m[3], double al, int d, double s, double n[3])
     return x;
 }
 
-// Flux through a face of the donor of fraction cv in (0, 1) with normal
-// direction m (largest component within 2^-20 .. 2^20); s is the signed
-// Courant number.
+// Flux through a face of the donor cut by the plane of direction m (largest
+// component within 2^-20 .. 2^20) and constant al in the reflected frame; s is
+// the signed Courant number.
+VOF_HD double face_flux64_at(const double m[3], double al, int d, double s) {
+    double n[3];
+    const double x = slab64(m, al, d, s, n);
+    if (!lt_pos(0.0, n[2])) return bits64(x) > 0 ? s : 0.0;
+    return s * vol64(n[0], n[1], n[2], x);
+}
+// The same for a donor of fraction cv in (0, 1).
 VOF_HD double face_flux64(const double m[3], double cv, int d, double s) {
     double a = abs64(m[0]), b = abs64(m[1]), c = abs64(m[2]);
     sort3_pos(a, b, c);
-    double n[3];
-    const double x = slab64(m, alpha64(a, b, c, cv), d, s, n);
-    if (!lt_pos(0.0, n[2])) return bits64(x) > 0 ? s : 0.0;
-    return s * vol64(n[0], n[1], n[2], x);
+    return face_flux64_at(m, alpha64(a, b, c, cv), d, s);
 }
 
 }  // namespace vof

@@ -72,6 +72,8 @@ def pattern(kind, rng, shape=(7, 9, 11)):
         c = 0.5 + 1e-6 * rng.standard_normal(shape)
     elif kind == "spread":  # sixteen decades
         c = 10.0 ** (-16.0 * rng.random(shape))
+    elif kind == "rounding":  # whole numbers of 2^-56 among zeros, norms of 1 to a few units in the last place
+        c = np.where(rng.random(shape) < 0.5, 0.0, rng.integers(1, 200, shape) * 2.0 ** -56)
     else:  # residues about the least norm at which the rule takes Youngs' normal
         c = 10.0 ** (-29.0 - 3.0 * rng.random(shape))
     return np.ascontiguousarray(c, dtype=np.float64)
@@ -84,7 +86,7 @@ def pattern(kind, rng, shape=(7, 9, 11)):
 # differences are 1e-6 of them).  A centred-column normal has a component 1.
 @pytest.mark.parametrize("kind, tol", [("diagonal", 1e-13), ("axis", 1e-13), ("sixteenths", 1e-13),
                                        ("mixed", 1e-13), ("flat", 1e-7), ("spread", 1e-13),
-                                       ("residue", 1e-13)])
+                                       ("residue", 1e-13), ("rounding", 1e-13)])
 def test_normal_direction(vof, kind, tol):
     c = pattern(kind, np.random.default_rng(5))
     cfg = vof.make_config(c.shape[2], c.shape[1], c.shape[0])
