@@ -116,8 +116,8 @@ Layout layout_for(const vof_config* c) {
     L.size[S_MISC] = kMiscBytes;
     L.size[S_BITS] = K * words * 4;
     L.size[S_CCBITS] = K * words * 4;
-    // maps of the words that may hold a non-zero value: of c, and of the two sweep buffers
-    L.size[S_NZ] = 3 * nz_map_bytes(words);
+    // maps of the words that may hold a non-zero value: of c, and of the two sweep buffers; of their end cells (two)
+    L.size[S_NZ] = 5 * nz_map_bytes(words);
     L.size[S_NCMAP] = K * words * 4;
     L.size[S_MVBITS] = K * words * 4;
     // Step 4: the active fields' and the moving drops' bits dilated, plus scratch
@@ -267,6 +267,7 @@ static BoxSet<T, 1> ctx_box_set(vof_ctx* ctx, double* clipped, double dt) {
     B.nzc = ctx->slot<uint16_t>(S_NZ);
     B.nz1 = B.nzc + map;
     B.nz2 = B.nz1 + map;
+    B.nze = reinterpret_cast<uint32_t*>(B.nz2 + map);
     B.clipped = clipped;
     S.n = 1;
     S.tw = tile_words(B.words);
@@ -455,7 +456,10 @@ vof_status recolour_impl(vof_ctx* ctx, int* moved_out, int* fired_out, SweepArgs
     VOF_CUDA(ctx, cudaMemcpyAsync(d_target, target.data(), (size_t)M * 4, cudaMemcpyHostToDevice, st));
     VOF_CUDA(ctx, timed(ctx, P_MOVE, [&] {
                  return recolour_move(ctx->cur, ctx->fp64, labels, ctx->slot<uint32_t>(S_MVBITS), g, mt, d_fields,
-                                     (int)hfields.size(), d_target, ctx->slot<uint16_t>(S_NZ), st);
+                                     (int)hfields.size(), d_target, ctx->slot<uint16_t>(S_NZ),
+                                     reinterpret_cast<uint32_t*>(ctx->slot<char>(S_NZ) +
+                                                                 3 * nz_map_bytes((size_t)g.rows * g.W)),
+                                     st);
              }));
     ctx->launches += 1;
     if (patch && moved > 0 && ctx->n_active != na0) {

@@ -71,11 +71,11 @@ BatchLayout batch_layout(const vof_batch_config* cfg, const vof_box_desc* boxes,
         words_all += (long long)words;
         entries += list_reserve((long long)words, d.k_capacity);
     }
-    // maps of the words that may hold a non-zero value, three per box
+    // maps of the words that may hold a non-zero value, three per box, and of their end cells (two maps' room)
     L.nz_maps = o;
     for (int b = 0; b < n; ++b) {
         const size_t words = (size_t)boxes[b].ny * boxes[b].nz * ((boxes[b].nx + 31) / 32);
-        L.nz.push_back(o), o += 3 * al256(words * sizeof(uint16_t));
+        L.nz.push_back(o), o += 5 * al256(words * sizeof(uint16_t));
     }
     L.nz_bytes = o - L.nz_maps;
     L.words = words_all;
@@ -143,6 +143,7 @@ BoxSet<T, kMaxBoxes> batch_set(vof_batch* B) {
         X.nzc = (uint16_t*)(B->ws + B->L.nz[b]);
         X.nz1 = X.nzc + map;
         X.nz2 = X.nz1 + map;
+        X.nze = reinterpret_cast<uint32_t*>(X.nz2 + map);
         S.tiles += (X.words + S.tw - 1) / S.tw;
     }
     return S;
@@ -379,6 +380,9 @@ vof_status vof_batch_tune(vof_batch* B) {
     B->update_blocks_per_sm = bp;
     B->tune_ms_best = best;
     B->tune_candidates = n;
+    // the timed sweeps used both lists and the maps: the next step lists afresh
+    B->list_valid = false;
+    B->list_cur = 0;
     // the timed sweeps counted faces: start the counters afresh
     if (cudaMemsetAsync(B->ws + B->L.misc + 8, 0, 24, B->stream) != cudaSuccess) return fail(B, VOF_ERR_CUDA);
     for (auto& r : B->graphs)

@@ -72,6 +72,8 @@ struct BoxDev {
     uint16_t* nzc;      // [rows][W] fields with a non-zero value in the word of c, of b1 and of b2
     uint16_t* nz1;      // (a set bit may stand for a word of zeros)
     uint16_t* nz2;
+    uint32_t* nze;      // [rows][W] fields non-zero in the word's first cell (low half) and last cell (high half)
+                        // of the state that the next sweep along x reads
     double* clipped;    // [K] volume removed by the clip
 };
 
@@ -199,7 +201,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_list_sp(const __grid_constant
                     nhi |= (valid && vsign(uh[e]) > 0 ? 1u : 0u) << e;
                 }
             }
-            uint32_t nz = 0;
+            uint32_t nz = 0, edge_lo = 0, edge_hi = 0;  // fields non-zero in the word, in the lane's first and last cell
             for (int f0 = 0; f0 < B.K; f0 += FB) {
                 T cv[FB][VW];
 #pragma unroll
@@ -221,6 +223,10 @@ __global__ void __launch_bounds__(kSweepThreads) k_list_sp(const __grid_constant
                     uint32_t ow = 0;
                     if (vote) {  // the same for the warp
                         if (vote & group) nz |= 1u << f;
+                        if (d == 0) {
+                            edge_lo |= (is_exact_zero(cv[q][0]) ? 0u : 1u) << f;
+                            edge_hi |= (is_exact_zero(cv[q][VW - 1]) ? 0u : 1u) << f;
+                        }
                         ow = gather_word<VW>(valid ? occ : 0u, lane);
                         const uint32_t fl = inter & nlo, fh = inter & nhi;
                         const int n = __popc(fl) + __popc(fh);
@@ -238,6 +244,11 @@ __global__ void __launch_bounds__(kSweepThreads) k_list_sp(const __grid_constant
                 }
             }
             if (ok && gl == 0) B.nzc[word] = (uint16_t)nz;
+            if (d == 0 && valid) {
+                uint16_t* const e16 = reinterpret_cast<uint16_t*>(B.nze + word);
+                if (gl == 0) e16[0] = (uint16_t)edge_lo;
+                if (i + VW == min(p.i0 + 32, g.nx)) e16[1] = (uint16_t)edge_hi;
+            }
         }
     }
     out.flush(lane);
@@ -253,14 +264,18 @@ __global__ void __launch_bounds__(kSweepThreads) k_list_sp(const __grid_constant
 // non-zero in the input, or when the output buffer may hold something there
 // that has to become zero; every other word is zero in both buffers and is
 // neither read nor written (drops fill a few per cent of a field: one word in
-// five is active at phi = 0.3 in 8 fields).  The block collects the tile's
+// five is active at phi = 0.3 in 8 fields).  Along x a neighbour word counts by
+// its cell next to this one alone: the pass (or listing) before a sweep along x
+// leaves a map of the words' end cells (without it two words in three that were
+// active there were so for nothing).  The block collects the tile's
 // active (word, field) items in shared memory, so that lane groups work on
 // full items whatever their pattern; items of a word follow each other, so
 // its velocities come from L1 after the first.
 //
 // Bound: latency (three dependent loads per item: map, values, listed flux).
 // 256^3, K = 8, phi = 0.3, FP32: 0.17 ms per y or z sweep (0.38 ms when every
-// word of every field was read and written), 0.28 ms per x sweep (0.43 ms).
+// word of every field was read and written), 0.16 ms per x sweep (0.43 ms; 0.28 ms
+// with whole neighbour words); FP64 0.68 to 0.79 ms.
 template <typename T, int NB, int VW, int PH, bool DX>
 __global__ void __launch_bounds__(kSweepThreads, 4)
     k_update_sp(const __grid_constant__ BoxSet<T, NB> S, int d, int dn, T tau,
@@ -273,6 +288,7 @@ __global__ void __launch_bounds__(kSweepThreads, 4)
     __shared__ uint16_t s_item[kTileWords * 16];  // word of the tile << 4 | field
     __shared__ uint16_t s_cc[kTileWords];         // fields that were non-zero at the step's start
     __shared__ uint32_t s_new[kTileWords];        // fields with a non-zero result
+    __shared__ uint32_t s_edge[DX ? 1 : kTileWords];  // the same of the word's first and last cell
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, gl = lane & (LPW - 1);
     const unsigned group = (0xffffffffu >> (32 - LPW)) << (lane & ~(LPW - 1));
     FaceWriter out(s_buf[warp], nlist, ncount);
@@ -288,9 +304,11 @@ __global__ void __launch_bounds__(kSweepThreads, 4)
             s_place[t0] = place_word(B, w0 + t0, d, dn, wlo, whi);
             const uint16_t* __restrict__ in = nz_in(B, PH);
             out_old = nz_out(B, PH)[w0 + t0];
-            act = ((uint32_t)in[w0 + t0] | in[wlo] | in[whi] | out_old) & ((1u << B.K) - 1u);
+            const uint32_t beside = DX ? B.nze[wlo] >> 16 | (B.nze[whi] & 0xffffu) : (uint32_t)in[wlo] | in[whi];
+            act = (in[w0 + t0] | beside | out_old) & ((1u << B.K) - 1u);
             if (PH > 0) s_cc[t0] = PH == 2 ? (uint16_t)out_old : B.nzc[w0 + t0];
             s_new[t0] = 0u;
+            if (!DX) s_edge[t0] = 0u;
         }
         // the tile's items, word by word
         const int cnt = __popc(act);
@@ -429,6 +447,10 @@ __global__ void __launch_bounds__(kSweepThreads, 4)
             if (valid) stv<VW>(sweep_out(B, PH) + (size_t)f * g.N + x, v);
             const unsigned vote = __ballot_sync(0xffffffffu, valid && nonzero);
             if (ok && gl == 0 && (vote & group)) atomicOr(&s_new[t], 1u << f);
+            if (!DX && dn == 0 && valid) {
+                if (gl == 0 && !is_exact_zero(v[0])) atomicOr(&s_edge[t], 1u << f);
+                if (i + VW == min(p.i0 + 32, g.nx) && !is_exact_zero(v[VW - 1])) atomicOr(&s_edge[t], 0x10000u << f);
+            }
             if (PH == 2) {
                 const uint32_t w = gather_word<VW>(occm, lane);
                 if (ok && gl == 0) B.occbits[word] = w;
@@ -457,9 +479,10 @@ __global__ void __launch_bounds__(kSweepThreads, 4)
         if (t0 < nw) {
             const uint32_t m = s_new[t0] | (out_old & ~((1u << B.K) - 1u));
             if (m != out_old) nz_out(B, PH)[w0 + t0] = (uint16_t)m;
+            if (!DX && dn == 0) B.nze[w0 + t0] = s_edge[t0];
         }
         // (the next tile's first barrier comes before anything reads what its
-        // build writes, and this thread's s_new is read above by itself)
+        // build writes, and this thread's s_new and s_edge are read above by itself)
     }
     out.flush(lane);
 }

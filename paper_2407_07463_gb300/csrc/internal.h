@@ -188,11 +188,12 @@ cudaError_t recolour_touch(const int* labels, const uint32_t* bits, uint32_t* mv
 // The bit map of moving tags (mt.mv_map, cleared by the caller) for the
 // n_fields fields listed in mv_fields.
 cudaError_t move_map(MoveTables mt, uint32_t* map, const int* mv_fields, int n_fields, cudaStream_t st);
-// Moves the cells set in mvbits to their drop's target field, whose bit of
-// the map of non-zero words (nzc, 16 bits per word) is set.
+// Moves the cells set in mvbits to their drop's target field, whose bits of
+// the maps of non-zero words (nzc, 16 bits per word) and end cells (nze, twice
+// 16 bits) are set.
 cudaError_t recolour_move(void* c, bool fp64, const int* labels, const uint32_t* mvbits, const Dims& g,
                           MoveTables mt, const int* mv_fields, int n_mv_fields, const int* target, uint16_t* nzc,
-                          cudaStream_t st);
+                          uint32_t* nze, cudaStream_t st);
 
 // Statistics helpers.
 // Drops of the slots' fields, counted slot after slot (a single field: one

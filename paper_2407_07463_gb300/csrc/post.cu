@@ -167,7 +167,8 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_move(T* c, const int* __restrict__ labels,
                                               const uint32_t* __restrict__ mvbits, Dims g, MoveTables mt,
                                               const int* __restrict__ mv_fields, int n_mv_fields,
-                                              const int* __restrict__ target, uint32_t* __restrict__ nzc) {
+                                              const int* __restrict__ target, uint32_t* __restrict__ nzc,
+                                              uint32_t* __restrict__ nze) {
     const long long per_field = (long long)g.rows * g.W;
     const long long words = (long long)n_mv_fields * per_field;
     for (long long wd = (long long)blockIdx.x * blockDim.x + threadIdx.x; wd < words;
@@ -192,7 +193,10 @@ __global__ void __launch_bounds__(256) k_move(T* c, const int* __restrict__ labe
             c[(size_t)f * g.N + x] = T(0);
             filled |= 1u << tg;
         }
-        if (filled) atomicOr(nzc + (rem >> 1), filled << (16 * (int)(rem & 1)));
+        if (filled) {
+            atomicOr(nzc + (rem >> 1), filled << (16 * (int)(rem & 1)));
+            atomicOr(nze + rem, filled * 0x10001u);  // (either end may be among them)
+        }
     }
 }
 
@@ -214,15 +218,15 @@ cudaError_t move_map(MoveTables mt, uint32_t* map, const int* mv_fields, int n_f
 
 cudaError_t recolour_move(void* c, bool fp64, const int* labels, const uint32_t* mvbits, const Dims& g,
                           MoveTables mt, const int* mv_fields, int n_mv_fields, const int* target, uint16_t* nzc,
-                          cudaStream_t st) {
+                          uint32_t* nze, cudaStream_t st) {
     const long long words = (long long)n_mv_fields * g.rows * g.W;
     uint32_t* nz = reinterpret_cast<uint32_t*>(nzc);
     if (fp64)
         k_move<double><<<grid_for(words, 256), 256, 0, st>>>((double*)c, labels, mvbits, g, mt, mv_fields,
-                                                            n_mv_fields, target, nz);
+                                                            n_mv_fields, target, nz, nze);
     else
         k_move<float><<<grid_for(words, 256), 256, 0, st>>>((float*)c, labels, mvbits, g, mt, mv_fields,
-                                                           n_mv_fields, target, nz);
+                                                           n_mv_fields, target, nz, nze);
     return cudaGetLastError();
 }
 

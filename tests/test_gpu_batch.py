@@ -129,3 +129,19 @@ def test_batch_argument_errors(vof, boxes):
         B.step(1)
     assert e.value.status == vof.VOF_ERR_STATE
     B.close()
+
+
+def test_batch_tuned_between_steps(vof, boxes):
+    """The timed sweeps use the face lists and maps of the running batch: the
+    steps after a tuning list their faces again."""
+    want = run_contexts(vof, boxes, 1, 5)
+    cs = [dev(w.c, torch.float32) for w in boxes]
+    us = [dev(w.u, torch.float32) for w in boxes]
+    B = vof.Batch(list(zip(cs, us, [w.dt for w in boxes])), precision=1, k_active=[w.k_active for w in boxes])
+    for n in (1, 2, 2):  # both lists and two directions have been current
+        B.step(n)
+        B.tune()
+    torch.cuda.synchronize()
+    for c, w in zip(cs, want):
+        assert np.array_equal(c.cpu().numpy(), w)
+    B.close()

@@ -121,3 +121,24 @@ def test_refined_faces(vof, shape, K, band):
     ctx.vof_step(dt, 1)
     assert np.abs(c_d.cpu().numpy() - want).max() <= 1e-5
     ctx.close()
+
+
+@pytest.mark.parametrize("nx", [32, 33, 64, 70])
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_words_entered_along_x(vof, nx, sign):
+    """Interfacial cells at the ends of words, carried along x into words that
+    hold nothing (also across the wrap, into a last word of one and six cells)."""
+    shape, K = (4, 4, nx), 3
+    c = np.zeros((K,) + shape)
+    rng = np.random.default_rng(nx)
+    for k, i in enumerate((0, 31, nx - 1)):
+        c[k, 1:3, 1:3, i] = 0.3 + 0.6 * rng.random((2, 2))
+    u = np.zeros((3,) + shape)
+    u[0], u[1], u[2] = sign, 0.31, -0.23
+    c_d = torch.from_numpy(c).to(DEV)
+    ctx = vof.Context(vof.make_config(nx, 4, 4, k_capacity=K, k_active=K, recolour=0), c_d,
+                      torch.from_numpy(u).to(DEV))
+    ctx.vof_step(0.4, 3)
+    want, _ = O.advect(c, u, 0.4, 1.0, 3)
+    assert np.abs(c_d.cpu().numpy() - want).max() <= 1e-12
+    ctx.close()
