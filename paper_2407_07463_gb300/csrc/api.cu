@@ -229,6 +229,7 @@ vof_status check_ctx(vof_ctx* ctx) {
 
 vof_status scan_velocity(vof_ctx* ctx) {
     double* vs = (double*)(ctx->misc() + kMiscVscan);
+    VOF_CUDA(ctx, cudaMemsetAsync(vs, 0, 2 * sizeof(double), ctx->stream));
     VOF_CUDA(ctx, velocity_scan(ctx->fp64, ctx->u, 3ll * ctx->g.N, vs, ctx->stream));
     ctx->launches += 1;
     unsigned long long host[2];

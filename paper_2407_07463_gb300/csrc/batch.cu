@@ -49,7 +49,7 @@ bool batch_config_valid(const vof_batch_config* c) {
 // Per-box slices and shared buffers of the batch workspace.
 struct BatchLayout {
     std::vector<size_t> b1, b2, flux, net, ccbits, occbits, nz;
-    size_t nz_maps, nz_bytes, clipped, list, counts, misc, vscan, total;
+    size_t nz_maps, nz_bytes, clipped, list, counts, misc, total;
     long long list_entries, words;
 };
 
@@ -84,7 +84,6 @@ BatchLayout batch_layout(const vof_batch_config* cfg, const vof_box_desc* boxes,
     L.list = o, o = al256(o + 2 * (size_t)L.list_entries * 8);
     L.counts = o, o = al256(o + 2 * sizeof(int));
     L.misc = o, o = al256(o + 64);  // [0] tensor-core status, [8..32) face counters
-    L.vscan = o, o = al256(o + 16);
     L.total = o;
     return L;
 }
@@ -317,20 +316,27 @@ vof_status vof_batch_init(const vof_batch_config* cfg, const vof_box_desc* boxes
     B->sticky = VOF_OK;
     // velocities: finite, and the time step of each box within CFL 1/2
     const bool fp64 = cfg->precision == VOF_FP64;
-    double* vs = (double*)(B->ws + B->L.vscan);
-    for (int b = 0; b < n_boxes; ++b) {
+    // (each box's result in its slots of the clip sums, which are zeroed below;
+    // one read for all boxes)
+    unsigned long long* vs = (unsigned long long*)(B->ws + B->L.clipped);
+    std::vector<unsigned long long> host((size_t)n_boxes * 16);
+    cudaError_t ve = cudaMemsetAsync(vs, 0, host.size() * 8, B->stream);
+    for (int b = 0; b < n_boxes && ve == cudaSuccess; ++b) {
         const vof_box_desc& d = boxes[b];
-        unsigned long long host[2];
-        if (velocity_scan(fp64, d.u_dev, 3ll * d.nx * d.ny * d.nz, vs, B->stream) != cudaSuccess ||
-            cudaMemcpyAsync(host, vs, sizeof(host), cudaMemcpyDeviceToHost, B->stream) != cudaSuccess ||
-            cudaStreamSynchronize(B->stream) != cudaSuccess) {
-            (void)cudaGetLastError();
-            delete B;
-            return VOF_ERR_CUDA;
-        }
+        ve = velocity_scan(fp64, d.u_dev, 3ll * d.nx * d.ny * d.nz, (double*)(vs + (size_t)b * 16), B->stream);
+    }
+    if (ve != cudaSuccess ||
+        cudaMemcpyAsync(host.data(), vs, host.size() * 8, cudaMemcpyDeviceToHost, B->stream) != cudaSuccess ||
+        cudaStreamSynchronize(B->stream) != cudaSuccess) {
+        (void)cudaGetLastError();
+        delete B;
+        return VOF_ERR_CUDA;
+    }
+    for (int b = 0; b < n_boxes; ++b) {
         double mx;
-        std::memcpy(&mx, &host[0], sizeof(double));
-        vof_status s = host[1] ? VOF_ERR_NONFINITE : (mx * d.dt / cfg->h > 0.5 ? VOF_ERR_CFL : VOF_OK);
+        std::memcpy(&mx, &host[(size_t)b * 16], sizeof(double));
+        const vof_status s = host[(size_t)b * 16 + 1] ? VOF_ERR_NONFINITE
+                                                      : (mx * boxes[b].dt / cfg->h > 0.5 ? VOF_ERR_CFL : VOF_OK);
         if (s != VOF_OK) {
             delete B;
             return s;

@@ -266,8 +266,8 @@ __global__ void __launch_bounds__(kSweepThreads) k_list_sp(const __grid_constant
 // neither read nor written (drops fill a few per cent of a field: one word in
 // five is active at phi = 0.3 in 8 fields).  Along x a neighbour word counts by
 // its cell next to this one alone: the pass (or listing) before a sweep along x
-// leaves a map of the words' end cells (without it two words in three that were
-// active there were so for nothing).  The block collects the tile's
+// leaves a map of the words' end cells (whole neighbour words made the sweep take
+// 1.7 times as long).  The block collects the tile's
 // active (word, field) items in shared memory, so that lane groups work on
 // full items whatever their pattern; items of a word follow each other, so
 // its velocities come from L1 after the first.

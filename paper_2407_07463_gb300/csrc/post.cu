@@ -5,6 +5,7 @@
 #include "common.cuh"
 #include "internal.h"
 #include "plic.cuh"
+#include "update_vec.cuh"
 
 namespace vof {
 
@@ -838,33 +839,62 @@ cudaError_t normals_field(bool fp64, const void* cf, const Dims& g, void* m, cud
     return cudaGetLastError();
 }
 
-// out2[0] = max |u|, out2[1] = 1 if any non-finite value (both as double).
-template <typename T>
-__global__ void k_vscan(const T* __restrict__ u, long long n, unsigned long long* __restrict__ out) {
-    double mx = 0.0;
+// out[0] = max |u| over the finite values, out[1] = 1 if any is not finite (both
+// zero before; the maximum as a double's bits).  Magnitudes order as their bit
+// patterns, so the pass runs on integers, 16 bytes a load where u allows it, and
+// a block adds one atomic: with one per warp the atomics on one address were
+// the time (32 boxes of 32^3 to 128^3 in turn: 0.63 -> 0.14 ms).
+template <typename T, typename I>
+__global__ void __launch_bounds__(256) k_vscan(const T* __restrict__ u, long long n, long long n_vec,
+                                               unsigned long long* __restrict__ out) {
+    constexpr I kMag = (I)~(I)0 >> 1, kInf = sizeof(T) == 8 ? (I)0x7ff0000000000000ULL : (I)0x7f800000U;
+    constexpr int W = 16 / sizeof(T);
+    __shared__ I s_mx[8];
+    __shared__ unsigned s_bad;
+    I mx = 0;
     unsigned bad = 0;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n;
-         t += (long long)gridDim.x * blockDim.x) {
-        double v = (double)u[t];
-        if (!isfinite(v)) bad = 1;
-        else mx = fmax(mx, fabs(v));
+    auto take = [&](T v) {
+        I b;
+        memcpy(&b, &v, sizeof(T));
+        b &= kMag;
+        if (b >= kInf) bad = 1;
+        else mx = b > mx ? b : mx;
+    };
+    const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+    for (long long t = first; t < n_vec; t += stride) {
+        T v[W];
+        ldv<W>(u + t * W, v);
+#pragma unroll
+        for (int e = 0; e < W; ++e) take(v[e]);
     }
+    for (long long t = n_vec * W + first; t < n; t += stride) take(u[t]);
+    if (threadIdx.x == 0) s_bad = 0u;
     for (int o = 16; o > 0; o >>= 1) {
-        mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, o));
-        bad |= __shfl_down_sync(0xffffffffu, bad, o);
+        const I other = __shfl_down_sync(0xffffffffu, mx, o);
+        mx = other > mx ? other : mx;
     }
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(out, (unsigned long long)__double_as_longlong(mx));  // non-negative doubles order as ints
-        if (bad) atomicOr(out + 1, 1ull);
-    }
+    if ((threadIdx.x & 31) == 0) s_mx[threadIdx.x >> 5] = mx;
+    __syncthreads();
+    if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(&s_bad, 1u);
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int w = 1; w < 8; ++w) mx = s_mx[w] > mx ? s_mx[w] : mx;
+    T v;
+    memcpy(&v, &mx, sizeof(T));
+    if (mx != 0) atomicMax(out, (unsigned long long)__double_as_longlong((double)v));
+    if (s_bad) atomicOr(out + 1, 1ull);
 }
 
 cudaError_t velocity_scan(bool fp64, const void* u, long long n, double* out2, cudaStream_t st) {
-    cudaMemsetAsync(out2, 0, 2 * sizeof(double), st);
+    const bool vec = ((uintptr_t)u & 15) == 0;
+    const long long n_vec = vec ? n / (fp64 ? 2 : 4) : 0;
+    // a few loads a thread: enough blocks for the memory, few atomics
+    const int blocks = (int)std::max(1ll, std::min<long long>(sm_count() * 8, (n + 2047) / 2048));
     if (fp64)
-        k_vscan<double><<<grid_for(n, 256), 256, 0, st>>>((const double*)u, n, (unsigned long long*)out2);
+        k_vscan<double, unsigned long long>
+            <<<blocks, 256, 0, st>>>((const double*)u, n, n_vec, (unsigned long long*)out2);
     else
-        k_vscan<float><<<grid_for(n, 256), 256, 0, st>>>((const float*)u, n, (unsigned long long*)out2);
+        k_vscan<float, unsigned><<<blocks, 256, 0, st>>>((const float*)u, n, n_vec, (unsigned long long*)out2);
     return cudaGetLastError();
 }
 

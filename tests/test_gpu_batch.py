@@ -145,3 +145,41 @@ def test_batch_tuned_between_steps(vof, boxes):
     for c, w in zip(cs, want):
         assert np.array_equal(c.cpu().numpy(), w)
     B.close()
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 1), (1, 2, 5), (3, 5, 33), (8, 16, 64)])
+@pytest.mark.parametrize("precision,shift", [(0, 0), (1, 0), (0, 1), (1, 1), (1, 2)])
+def test_velocity_check(vof, shape, precision, shift):
+    """The largest |u| and a non-finite u found wherever they lie, with buffers
+    on and off a 16-byte boundary; in a batch, whichever box holds them."""
+    dt_ = torch.float64 if precision == 0 else torch.float32
+    n = 3 * shape[0] * shape[1] * shape[2]
+
+    def box(pos=None, value=0.0):
+        u = torch.zeros(n + shift, dtype=dt_, device=DEV)[shift:].view((3,) + shape)
+        u.fill_(-0.25)
+        if pos is not None:
+            u.view(-1)[pos] = value
+        return torch.zeros((1,) + shape, dtype=dt_, device=DEV), u, 1.0
+
+    def status(*boxes):
+        try:
+            if len(boxes) == 1:
+                c, u, dt = boxes[0]
+                ctx = vof.Context(vof.make_config(shape[2], shape[1], shape[0], precision=precision), c, u)
+                ctx.vof_step(dt, 1)
+                ctx.close()
+            else:
+                vof.Batch(list(boxes), precision=precision).close()
+        except vof.VofError as e:
+            return e.status
+        return 0
+
+    in_batch = shift == 0 and shape[2] % 4 == 0
+    assert status(box()) == 0
+    for pos in sorted({0, 1, n // 2, n - 2, n - 1}):
+        for value, want in ((-0.4375, 0), (0.5, 0), (-0.5625, vof.VOF_ERR_CFL), (float("nan"), vof.VOF_ERR_NONFINITE),
+                            (float("inf"), vof.VOF_ERR_NONFINITE), (-float("inf"), vof.VOF_ERR_NONFINITE)):
+            assert status(box(pos, value)) == want
+            if in_batch:
+                assert status(box(pos, value), box()) == want and status(box(), box(pos, value)) == want
