@@ -663,7 +663,8 @@ def run_ours(args, rank, world):
         if name == "update":
             own = algorithmic_bytes("update", N, fields, es)
             roof_update = dict(r, algorithmic_bytes_per_launch=own, achieved=own / (tot / cnt * 1e-3) / 1e9,
-                               basis="the update pass's own bytes per sweep (c in and out, bits, velocities)")
+                               basis="bytes of a pass over every word (c in and out, bits, velocities); "
+                                     "words that cannot change are skipped: an equivalent rate, not traffic")
             roof_update["frac"] = roof_update["achieved"] / hbm
         if name == "face_flux" and prec == vof.VOF_MIXED_LEARNED:
             roof_alu = alu_roofline(cnt, tot, rep, sm_count, sm_mhz)

@@ -429,7 +429,7 @@ const char *vof_profile_class_name(int32_t cls);
  * Each pass of a sweep is one launch covering every field of every box; a
  * step is replayed from a captured CUDA graph (one graph per sweep rotation
  * and list parity, captured on first use); the launch shape of the update
- * pass (warps per block, resident blocks per SM) is chosen by timing the
+ * pass (resident blocks per SM) is chosen by timing the
  * candidates on the batch's own first sweep (vof_batch_tune, run by the
  * first vof_batch_step when cfg.autotune is set).  The library allocates
  * nothing: the caller passes one device workspace.
@@ -459,7 +459,7 @@ typedef struct {
     double clipped_volume[64];     /* per box, accumulated since init */
     int64_t faces_network, faces_myc; /* VOF_MIXED_LEARNED, accumulated */
     int64_t faces_myc_judged;      /* faces whose MYC residual was evaluated */
-    int32_t update_warps, update_blocks_per_sm; /* launch shape in use */
+    int32_t update_warps, update_blocks_per_sm; /* launch shape in use (8 warps per block) */
     int32_t tune_candidates;       /* shapes timed by the tuner (0: not tuned) */
     float tune_best_ms;            /* median first-sweep time of the chosen shape */
     int64_t graph_launches, direct_steps;
@@ -478,8 +478,8 @@ vof_status vof_batch_init(const vof_batch_config *cfg, const vof_box_desc *boxes
                           void *workspace_dev, size_t workspace_bytes, void *stream, vof_batch **out);
 /* Learned normal for a VOF_MIXED_LEARNED batch (as vof_set_mlp). */
 vof_status vof_batch_set_mlp(vof_batch *batch, const void *weights_dev, double fallback_tol);
-/* Times the update launch shapes on the batch's first sweep (the state is
- * not modified) and keeps the fastest. */
+/* Times the update launch shapes on the batch's next sweep (the state is
+ * not modified) and keeps the fastest; the next step lists its faces afresh. */
 vof_status vof_batch_tune(vof_batch *batch);
 /* nsteps steps of every box, asynchronous on the batch's stream. */
 vof_status vof_batch_step(vof_batch *batch, int32_t nsteps);

@@ -101,7 +101,7 @@ void face_fluxes(const BoxSet<T, NB>& S, int d, int sweep, const unsigned long l
 }
 
 // nsteps steps of every box of S (Section 2.2 split advection with the
-// Weymouth & Yue term; c_c bits, clip and occupancy bits as in k_update).
+// Weymouth & Yue term; c_c bits, clip and occupancy bits as in k_update_sp).
 template <typename T, int NB>
 cudaError_t advect_set(const BoxSet<T, NB>& S, SweepArgs& a, int nsteps) {
     if (S.n == 0 || nsteps <= 0) return cudaSuccess;

@@ -145,7 +145,7 @@ __device__ __forceinline__ long long warp_append(bool flag, unsigned long long* 
     return (long long)(base + __popc(mask & ((1u << lane) - 1u)));
 }
 
-// Warp-aggregated append of nflag entries per lane to the block's segment;
+// Warp-aggregated append of nflag entries per lane to a block's list;
 // returns the lane's first slot.
 __device__ __forceinline__ int warp_reserve(int nflag, int lane, int* s_count) {
     int incl = nflag;
