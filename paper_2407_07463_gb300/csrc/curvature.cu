@@ -121,7 +121,9 @@ __global__ void __launch_bounds__(kCurvThreads) k_curvature(const T* __restrict_
     const T* __restrict__ cf = c + (size_t)blockIdx.y * g.N;
     T* __restrict__ kf = kappa + (size_t)blockIdx.y * g.N;
     const int lane = threadIdx.x & 31;
-    for (int base = blockIdx.x * kCurvTile; base < g.N; base += gridDim.x * kCurvTile) {
+    // (unsigned: a grid's stride past the last cell of 2^31 stays below 2^32)
+    for (unsigned start = blockIdx.x * kCurvTile; start < (unsigned)g.N; start += gridDim.x * kCurvTile) {
+        const int base = (int)start;
         if (threadIdx.x == 0) s_n = 0;
         __syncthreads();
         const int end = min(kCurvTile, g.N - base);  // a multiple of VW
@@ -166,8 +168,8 @@ __global__ void __launch_bounds__(kCurvThreads) k_curvature(const T* __restrict_
 template <typename T, int VW>
 __global__ void __launch_bounds__(256) k_surface_tension(const T* __restrict__ c, const T* __restrict__ kappa, int K,
                                                          Dims g, T h, T gamma, T* __restrict__ f) {
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < g.N / VW; t += gridDim.x * blockDim.x) {
-        const int x = t * VW;
+    for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < (unsigned)g.N / VW; t += gridDim.x * blockDim.x) {
+        const int x = (int)t * VW;
         int i, j, k;
         decode(x, g, i, j, k);
         const int xp = i == 0 ? x + g.nx - 1 : x - 1;  // the cell before the thread's first
