@@ -11,6 +11,8 @@ cudaError_t advect_set_fp32(const BoxSet<float, kMaxBoxes>& S, SweepArgs& a, int
 int update_occupancy(bool fp64) {
     return fp64 ? update_occupancy_fp64() : update_blocks_per_sm<float, kMaxBoxes, VecOf<float>::W>();
 }
+cudaError_t clear_set_fp32(const BoxSet<float, 1>& S, cudaStream_t st) { return clear_set(S, st); }
+cudaError_t clear_set_fp32(const BoxSet<float, kMaxBoxes>& S, cudaStream_t st) { return clear_set(S, st); }
 cudaError_t advect_first_sweep_fp32(const BoxSet<float, kMaxBoxes>& S, SweepArgs& a) {
     return advect_first_sweep(S, a);
 }

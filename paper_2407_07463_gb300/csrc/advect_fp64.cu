@@ -9,6 +9,8 @@ cudaError_t advect_set_fp64(const BoxSet<double, kMaxBoxes>& S, SweepArgs& a, in
     return advect_set(S, a, nsteps);
 }
 int update_occupancy_fp64() { return update_blocks_per_sm<double, kMaxBoxes, VecOf<double>::W>(); }
+cudaError_t clear_set_fp64(const BoxSet<double, 1>& S, cudaStream_t st) { return clear_set(S, st); }
+cudaError_t clear_set_fp64(const BoxSet<double, kMaxBoxes>& S, cudaStream_t st) { return clear_set(S, st); }
 cudaError_t advect_first_sweep_fp64(const BoxSet<double, kMaxBoxes>& S, SweepArgs& a) {
     return advect_first_sweep(S, a);
 }

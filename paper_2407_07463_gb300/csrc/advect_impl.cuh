@@ -80,6 +80,14 @@ bool lists_fit(const BoxSet<T, NB>& S, const SweepArgs& a) {
     return need <= a.list_entries;
 }
 
+// Sweep buffers and maps before the first step.
+template <typename T, int NB>
+cudaError_t clear_set(const BoxSet<T, NB>& S, cudaStream_t st) {
+    if (S.tiles <= 0) return cudaSuccess;
+    k_clear_sp<T, NB><<<std::min(S.tiles, sm_count() * 8), kSweepThreads, 0, st>>>(S);
+    return cudaGetLastError();
+}
+
 template <typename T, int NB>
 void face_fluxes(const BoxSet<T, NB>& S, int d, int sweep, const unsigned long long* list, const int* count,
                  int* next_count, SweepArgs& a) {

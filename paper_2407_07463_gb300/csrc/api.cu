@@ -604,8 +604,8 @@ vof_status vof_init(const vof_config* cfg, void* c_dev, const void* u_dev, void*
     ctx->mlp = nullptr;
     ctx->mlp_tol = 1e-3;
     if (cudaMemsetAsync(ctx->ws + L.off[S_MISC], 0, kMiscBytes, ctx->stream) != cudaSuccess ||
-        // the sweep buffers hold anything: every word may be non-zero
-        cudaMemsetAsync(ctx->ws + L.off[S_NZ], 0xff, L.size[S_NZ], ctx->stream) != cudaSuccess ||
+        (ctx->fp64 ? clear_set_fp64(ctx_box_set<double>(ctx, nullptr, 0.0), ctx->stream)
+                   : clear_set_fp32(ctx_box_set<float>(ctx, nullptr, 0.0), ctx->stream)) != cudaSuccess ||
         cudaMemsetAsync(ctx->ws + L.off[S_HIST_R], 0, L.size[S_HIST_R], ctx->stream) != cudaSuccess ||
         cudaMemsetAsync(ctx->ws + L.off[S_HIST_RT], 0, L.size[S_HIST_RT], ctx->stream) != cudaSuccess ||
         cudaMemsetAsync(ctx->ws + L.off[S_MOM], 0, L.size[S_MOM], ctx->stream) != cudaSuccess) {

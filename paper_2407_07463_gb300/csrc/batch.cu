@@ -49,7 +49,7 @@ bool batch_config_valid(const vof_batch_config* c) {
 // Per-box slices and shared buffers of the batch workspace.
 struct BatchLayout {
     std::vector<size_t> b1, b2, flux, net, ccbits, occbits, nz;
-    size_t nz_maps, nz_bytes, clipped, list, counts, misc, total;
+    size_t clipped, list, counts, misc, total;
     long long list_entries, words;
 };
 
@@ -72,12 +72,10 @@ BatchLayout batch_layout(const vof_batch_config* cfg, const vof_box_desc* boxes,
         entries += list_reserve((long long)words, d.k_capacity);
     }
     // maps of the words that may hold a non-zero value, three per box, and of their end cells (two maps' room)
-    L.nz_maps = o;
     for (int b = 0; b < n; ++b) {
         const size_t words = (size_t)boxes[b].ny * boxes[b].nz * ((boxes[b].nx + 31) / 32);
         L.nz.push_back(o), o += 5 * al256(words * sizeof(uint16_t));
     }
-    L.nz_bytes = o - L.nz_maps;
     L.words = words_all;
     L.list_entries = entries;
     L.clipped = o, o = al256(o + (size_t)n * 16 * 8);
@@ -342,8 +340,8 @@ vof_status vof_batch_init(const vof_batch_config* cfg, const vof_box_desc* boxes
             return s;
         }
     }
-    // the sweep buffers hold anything: every word may be non-zero
-    if (cudaMemsetAsync(B->ws + B->L.nz_maps, 0xff, B->L.nz_bytes, B->stream) != cudaSuccess ||
+    if ((fp64 ? clear_set_fp64(batch_set<double>(B), B->stream) : clear_set_fp32(batch_set<float>(B), B->stream)) !=
+            cudaSuccess ||
         cudaMemsetAsync(B->ws + B->L.clipped, 0, (size_t)n_boxes * 16 * 8, B->stream) != cudaSuccess ||
         cudaMemsetAsync(B->ws + B->L.misc, 0, 64, B->stream) != cudaSuccess) {
         (void)cudaGetLastError();

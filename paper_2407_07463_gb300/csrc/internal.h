@@ -93,6 +93,11 @@ cudaError_t patch_list_fp64(const BoxSet<double, 1>& S, SweepArgs& a, int d, con
 // asked of the unit that launches it.
 int update_occupancy(bool fp64);
 int update_occupancy_fp64();
+// Sweep buffers (the active fields) and their maps before the first step of a set.
+cudaError_t clear_set_fp64(const BoxSet<double, 1>& S, cudaStream_t st);
+cudaError_t clear_set_fp32(const BoxSet<float, 1>& S, cudaStream_t st);
+cudaError_t clear_set_fp64(const BoxSet<double, kMaxBoxes>& S, cudaStream_t st);
+cudaError_t clear_set_fp32(const BoxSet<float, kMaxBoxes>& S, cudaStream_t st);
 // Listing and first sweep of a batch only (state untouched; for timing).
 cudaError_t advect_first_sweep_fp64(const BoxSet<double, kMaxBoxes>& S, SweepArgs& a);
 cudaError_t advect_first_sweep_fp32(const BoxSet<float, kMaxBoxes>& S, SweepArgs& a);
