@@ -672,7 +672,7 @@ __global__ void __launch_bounds__(kFaceTile) k_face_flux_bx(const __grid_constan
             gather_stencil_ijk(sweep_in(B, sweep) + (size_t)fc.f * B.g.N, fc.di, fc.dj, fc.dk, B.g, st);
             cv = st[13];
             if constexpr (kBanded) myc_normal(st, m);
-            else myc_direction64(st, m);
+            else myc_direction64(st, m, kFluxEdge);
         }
         if constexpr (kBanded) {
             const bool queue = valid && (cv < band || cv > T(1) - band);
