@@ -109,6 +109,20 @@ __device__ __forceinline__ bool interfacial(double v) {  // the open interval on
     return b > 0 && b < 0x3FF0000000000000LL;
 }
 
+// 0 or 1: between two such cells nothing is added, whatever their neighbours are.
+__device__ __forceinline__ bool settled(float v) { return v == 0.f || v == 1.f; }
+__device__ __forceinline__ bool settled(double v) {
+    const long long b = __double_as_longlong(v);
+    return b << 1 == 0 || b == 0x3FF0000000000000LL;
+}
+// acc + zero * (p - q), zero being 0 (or a NaN): changes acc only where the
+// difference is not finite.  In double without FP64 instructions elsewhere.
+__device__ __forceinline__ void add_nothing(float& acc, float zero, float p, float q) { acc += zero * (p - q); }
+__device__ __forceinline__ void add_nothing(double& acc, double zero, double p, double q) {
+    const int big = max(__double2hiint(p) & 0x7fffffff, __double2hiint(q) & 0x7fffffff);
+    if (big >= 0x7fd00000 || !is_exact_zero(zero)) acc += zero * (p - q);  // (below 2^1022 a difference is finite)
+}
+
 // Curvatures of the fields blockIdx.y of c ([K][N]) into kappa: NaN in every
 // cell without one if FILL, else only the interfacial cells are written.
 constexpr int kCurvThreads = 256, kCurvTile = 8192;
@@ -163,11 +177,14 @@ __global__ void __launch_bounds__(kCurvThreads) k_curvature(const T* __restrict_
 // f[d][x] on the low d-face of cell x: sum over the K fields of
 // gamma kappa_f (c(x) - c(x - e_d)) / h, kappa_f the mean of the two cells'
 // curvatures where both have one, else the one that does, else 0.  Only an
-// interfacial cell can have a curvature (kappa holds nothing elsewhere).  A
-// thread takes VW cells of a row.
+// interfacial cell can have a curvature (kappa holds nothing elsewhere).  Faces
+// without a curvature add 0 and are left out, except where 0 times the rest is not
+// 0: a NaN or an infinity in c reaches the faces beside it.  A thread takes VW
+// cells of a row.
 template <typename T, int VW>
-__global__ void __launch_bounds__(256) k_surface_tension(const T* __restrict__ c, const T* __restrict__ kappa, int K,
+__global__ void __launch_bounds__(256, 4) k_surface_tension(const T* __restrict__ c, const T* __restrict__ kappa, int K,
                                                          Dims g, T h, T gamma, T* __restrict__ f) {
+    const T zero = gamma * T(0) / h;  // a NaN for gamma or h beyond the range of T
     for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < (unsigned)g.N / VW; t += gridDim.x * blockDim.x) {
         const int x = (int)t * VW;
         int i, j, k;
@@ -189,11 +206,11 @@ __global__ void __launch_bounds__(256) k_surface_tension(const T* __restrict__ c
             ldv<VW>(cq + x + ly, cl[1]);
             ldv<VW>(cq + x + lz, cl[2]);
             const T cp = cq[xp];
-            bool any = interfacial(cp);
+            bool any = !(settled(cp) && is_exact_zero(zero));
 #pragma unroll
             for (int e = 0; e < VW; ++e) {
                 cl[0][e] = e == 0 ? cp : cr[e == 0 ? 0 : e - 1];
-                any = any || interfacial(cr[e]) || interfacial(cl[1][e]) || interfacial(cl[2][e]);
+                any = any || !(settled(cr[e]) && settled(cl[1][e]) && settled(cl[2][e]));
             }
             if (!any) continue;
 #pragma unroll
@@ -204,7 +221,10 @@ __global__ void __launch_bounds__(256) k_surface_tension(const T* __restrict__ c
                 for (int d = 0; d < 3; ++d) {
                     const T kl = interfacial(cl[d][e]) ? kq[xl[d]] : nan_of<T>();
                     const bool fl = isfinite(kl), fr = isfinite(kr);
-                    if (!fl && !fr) continue;
+                    if (!fl && !fr) {
+                        add_nothing(acc[d][e], zero, cr[e], cl[d][e]);
+                        continue;
+                    }
                     const T kf = fl && fr ? T(0.5) * (kl + kr) : (fl ? kl : kr);
                     acc[d][e] += gamma * kf * (cr[e] - cl[d][e]) / h;
                 }
