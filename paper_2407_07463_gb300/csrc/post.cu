@@ -310,7 +310,7 @@ template <typename T, DropMode MODE>
 __device__ __forceinline__ void add_run(const T* __restrict__ cf, const Dims& g, const DropOut& o, int idx, int x, int i,
                                         int j, int k, int cnt, const RunSums<T>& rs) {
     if (MODE == DropRoots) {
-        atomicMin(o.root + idx, x);
+        atomicMin(reinterpret_cast<unsigned*>(o.root) + idx, (unsigned)x);
     } else if (MODE == DropSums) {
         int ri, rj, rk;
         decode(o.root[idx], g, ri, rj, rk);
@@ -484,7 +484,8 @@ static void launch_drop_words(const DropFields& D, const Dims& g, const DropOut&
 
 cudaError_t drop_roots(const DropFields& D, const Dims& g, int* root_of, cudaStream_t st) {
     if (D.n_max <= 0) return cudaSuccess;
-    const cudaError_t e = cudaMemsetAsync(root_of, 0x7f, (size_t)D.n_max * 4, st);
+    // above every cell's index as an unsigned number
+    const cudaError_t e = cudaMemsetAsync(root_of, 0xff, (size_t)D.n_max * 4, st);
     if (e != cudaSuccess) return e;
     launch_drop_words<DropRoots>(D, g, DropOut{root_of, nullptr, nullptr, nullptr, 0.0}, st);
     return cudaGetLastError();
