@@ -125,24 +125,24 @@ __device__ __forceinline__ void add_nothing(double& acc, double zero, double p, 
 
 // Curvatures of the fields blockIdx.y of c ([K][N]) into kappa: NaN in every
 // cell without one if FILL, else only the interfacial cells are written.
-constexpr int kCurvThreads = 256, kCurvTile = 8192;
+constexpr int kCurvThreads = 256;
 
-template <typename T, int VW, bool FILL>
+template <typename T, int VW, bool FILL, int TILE>
 __global__ void __launch_bounds__(kCurvThreads) k_curvature(const T* __restrict__ c, Dims g, T h,
                                                             T* __restrict__ kappa) {
-    __shared__ uint16_t s_cell[kCurvTile];
+    __shared__ uint16_t s_cell[TILE];
     __shared__ int s_n;
     const T* __restrict__ cf = c + (size_t)blockIdx.y * g.N;
     T* __restrict__ kf = kappa + (size_t)blockIdx.y * g.N;
     const int lane = threadIdx.x & 31;
     // (unsigned: a grid's stride past the last cell of 2^31 stays below 2^32)
-    for (unsigned start = blockIdx.x * kCurvTile; start < (unsigned)g.N; start += gridDim.x * kCurvTile) {
+    for (unsigned start = blockIdx.x * TILE; start < (unsigned)g.N; start += gridDim.x * TILE) {
         const int base = (int)start;
         if (threadIdx.x == 0) s_n = 0;
         __syncthreads();
-        const int end = min(kCurvTile, g.N - base);  // a multiple of VW
+        const int end = min(TILE, g.N - base);  // a multiple of VW
 #pragma unroll 4
-        for (int o = threadIdx.x * VW; o < kCurvTile; o += kCurvThreads * VW) {
+        for (int o = threadIdx.x * VW; o < TILE; o += kCurvThreads * VW) {
             T v[VW];
             uint32_t m = 0;
             if (o < end) {
@@ -241,11 +241,25 @@ static bool whole_lanes(const Dims& g, const void* p, const void* q) {
     return g.nx % VecOf<T>::W == 0 && (((uintptr_t)p | (uintptr_t)q) & 15) == 0;
 }
 
+template <typename T, bool FILL, int TILE>
+static void curvature_tiles(const T* c, int K, const Dims& g, T h, T* kappa, cudaStream_t st) {
+    const dim3 grid(grid_for(g.N, TILE, std::max(1, sm_count() * 32 / K)), K);
+    if (whole_lanes<T>(g, c, kappa))
+        k_curvature<T, VecOf<T>::W, FILL, TILE><<<grid, kCurvThreads, 0, st>>>(c, g, h, kappa);
+    else
+        k_curvature<T, 1, FILL, TILE><<<grid, kCurvThreads, 0, st>>>(c, g, h, kappa);
+}
+// Tiles of fewer cells while they are too few to give every SM four blocks: a
+// tile's interfacial cells are a block's serial work (every cell interfacial in
+// double: 16^3 took 128 us in tiles of 8192 and takes 19 now, 64^3 246 and 58; drops in
+// 28^3 72 and 22).  Half and twice as many blocks: 75 x 90 x 101 takes 17% and 21%
+// longer in FP32.
 template <typename T, bool FILL>
 static void curvature_launch(const T* c, int K, const Dims& g, T h, T* kappa, cudaStream_t st) {
-    const dim3 grid(grid_for(g.N, kCurvTile, std::max(1, sm_count() * 32 / K)), K);
-    if (whole_lanes<T>(g, c, kappa)) k_curvature<T, VecOf<T>::W, FILL><<<grid, kCurvThreads, 0, st>>>(c, g, h, kappa);
-    else k_curvature<T, 1, FILL><<<grid, kCurvThreads, 0, st>>>(c, g, h, kappa);
+    const long long cells = (long long)g.N * K / (4 * sm_count());
+    if (cells >= 8192) curvature_tiles<T, FILL, 8192>(c, K, g, h, kappa, st);
+    else if (cells >= 1024) curvature_tiles<T, FILL, 2048>(c, K, g, h, kappa, st);
+    else curvature_tiles<T, FILL, 256>(c, K, g, h, kappa, st);
 }
 
 template <typename T>
