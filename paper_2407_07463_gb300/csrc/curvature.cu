@@ -25,6 +25,7 @@
 // curvatures (few lanes of a warp gathering, an index modulo per value) and
 // 0.40 ms for the source.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "internal.h"
@@ -109,18 +110,32 @@ __device__ __forceinline__ bool interfacial(double v) {  // the open interval on
     return b > 0 && b < 0x3FF0000000000000LL;
 }
 
-// 0 or 1: between two such cells nothing is added, whatever their neighbours are.
-__device__ __forceinline__ bool settled(float v) { return v == 0.f || v == 1.f; }
-__device__ __forceinline__ bool settled(double v) {
-    const long long b = __double_as_longlong(v);
-    return b << 1 == 0 || b == 0x3FF0000000000000LL;
-}
+// Whether a value other than 0 and 1 is among those seen: between two such cells
+// nothing is added, whatever their neighbours are.  (In double by words: the low
+// ones join in one word, two to an instruction.)
+struct Unsettled32 {
+    bool any;
+    __device__ __forceinline__ void see(float v) { any = any || !(v == 0.f || v == 1.f); }
+    __device__ __forceinline__ bool found() const { return any; }
+};
+struct Unsettled64 {
+    bool any;
+    int low = 0;
+    __device__ __forceinline__ void see(double v) {
+        const int hi = __double2hiint(v);
+        low |= __double2loint(v);
+        any = any || !(hi == 0 || hi == 0x3FF00000);
+    }
+    __device__ __forceinline__ bool found() const { return any || low != 0; }
+};
+// v is finite (in double without an FP64 compare).
+__device__ __forceinline__ bool finite_bits(float v) { return isfinite(v); }
+__device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7FF00000) != 0x7FF00000; }
 // acc + zero * (p - q), zero being 0 (or a NaN): changes acc only where the
-// difference is not finite.  In double without FP64 instructions elsewhere.
-__device__ __forceinline__ void add_nothing(float& acc, float zero, float p, float q) { acc += zero * (p - q); }
-__device__ __forceinline__ void add_nothing(double& acc, double zero, double p, double q) {
-    const int big = max(__double2hiint(p) & 0x7fffffff, __double2hiint(q) & 0x7fffffff);
-    if (big >= 0x7fd00000 || !is_exact_zero(zero)) acc += zero * (p - q);  // (below 2^1022 a difference is finite)
+// difference is not finite.  In double a difference below 2^1023 is.
+__device__ __forceinline__ void add_nothing(float& acc, float zero, bool, float p, float q) { acc += zero * (p - q); }
+__device__ __forceinline__ void add_nothing(double& acc, double zero, bool all, double p, double q) {
+    if (all || max(__double2hiint(p) & 0x7FFFFFFF, __double2hiint(q) & 0x7FFFFFFF) >= 0x7FD00000) acc += zero * (p - q);
 }
 
 // Curvatures of the fields blockIdx.y of c ([K][N]) into kappa: NaN in every
@@ -179,12 +194,12 @@ __global__ void __launch_bounds__(kCurvThreads) k_curvature(const T* __restrict_
 // curvatures where both have one, else the one that does, else 0.  Only an
 // interfacial cell can have a curvature (kappa holds nothing elsewhere).  Faces
 // without a curvature add 0 and are left out, except where 0 times the rest is not
-// 0: a NaN or an infinity in c reaches the faces beside it.  A thread takes VW
-// cells of a row.
+// 0: a NaN or an infinity in c reaches the faces beside it.  zero: gamma * 0 / h,
+// a NaN for a gamma or h beyond the range of T.  A thread takes VW cells of a row.
 template <typename T, int VW>
 __global__ void __launch_bounds__(256, 4) k_surface_tension(const T* __restrict__ c, const T* __restrict__ kappa, int K,
-                                                         Dims g, T h, T gamma, T* __restrict__ f) {
-    const T zero = gamma * T(0) / h;  // a NaN for gamma or h beyond the range of T
+                                                         Dims g, T h, T gamma, T zero, T* __restrict__ f) {
+    const bool all_faces = !is_exact_zero(zero);
     for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < (unsigned)g.N / VW; t += gridDim.x * blockDim.x) {
         const int x = (int)t * VW;
         int i, j, k;
@@ -206,13 +221,16 @@ __global__ void __launch_bounds__(256, 4) k_surface_tension(const T* __restrict_
             ldv<VW>(cq + x + ly, cl[1]);
             ldv<VW>(cq + x + lz, cl[2]);
             const T cp = cq[xp];
-            bool any = !(settled(cp) && is_exact_zero(zero));
+            std::conditional_t<sizeof(T) == 8, Unsettled64, Unsettled32> u{all_faces};
+            u.see(cp);
 #pragma unroll
             for (int e = 0; e < VW; ++e) {
                 cl[0][e] = e == 0 ? cp : cr[e == 0 ? 0 : e - 1];
-                any = any || !(settled(cr[e]) && settled(cl[1][e]) && settled(cl[2][e]));
+                u.see(cr[e]);
+                u.see(cl[1][e]);
+                u.see(cl[2][e]);
             }
-            if (!any) continue;
+            if (!u.found()) continue;
 #pragma unroll
             for (int e = 0; e < VW; ++e) {
                 const T kr = interfacial(cr[e]) ? kq[x + e] : nan_of<T>();
@@ -220,9 +238,9 @@ __global__ void __launch_bounds__(256, 4) k_surface_tension(const T* __restrict_
 #pragma unroll
                 for (int d = 0; d < 3; ++d) {
                     const T kl = interfacial(cl[d][e]) ? kq[xl[d]] : nan_of<T>();
-                    const bool fl = isfinite(kl), fr = isfinite(kr);
+                    const bool fl = finite_bits(kl), fr = finite_bits(kr);
                     if (!fl && !fr) {
-                        add_nothing(acc[d][e], zero, cr[e], cl[d][e]);
+                        add_nothing(acc[d][e], zero, all_faces, cr[e], cl[d][e]);
                         continue;
                     }
                     const T kf = fl && fr ? T(0.5) * (kl + kr) : (fl ? kl : kr);
@@ -264,10 +282,12 @@ static void curvature_launch(const T* c, int K, const Dims& g, T h, T* kappa, cu
 
 template <typename T>
 static void tension_launch(const T* c, const T* kappa, int K, const Dims& g, T h, T gamma, T* f, cudaStream_t st) {
+    const T zero = gamma * T(0) / h;
     if (whole_lanes<T>(g, c, f))
-        k_surface_tension<T, VecOf<T>::W><<<grid_for(g.N / VecOf<T>::W, 256), 256, 0, st>>>(c, kappa, K, g, h, gamma, f);
+        k_surface_tension<T, VecOf<T>::W>
+            <<<grid_for(g.N / VecOf<T>::W, 256), 256, 0, st>>>(c, kappa, K, g, h, gamma, zero, f);
     else
-        k_surface_tension<T, 1><<<grid_for(g.N, 256), 256, 0, st>>>(c, kappa, K, g, h, gamma, f);
+        k_surface_tension<T, 1><<<grid_for(g.N, 256), 256, 0, st>>>(c, kappa, K, g, h, gamma, zero, f);
 }
 
 // Curvatures of K consecutive fields; fill: NaN in every cell without one.
