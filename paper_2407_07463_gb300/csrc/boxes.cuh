@@ -126,6 +126,14 @@ inline int tile_words(long long words) {
     return tw;
 }
 
+// A donor that is not empty.  An FP32 NaN counts as interfacial where a lane
+// takes one cell (rows that are not whole lanes), and spreads with the flux; where
+// it takes several it counts as empty, and stays in its cell.
+template <int VW, typename T>
+__device__ __forceinline__ bool holds(T v) {
+    return VW == 1 ? vclass(v) != 0 : above_zero(v);
+}
+
 // Place of one word of a tile.
 struct WordPlace {
     int x0, i0;               // first cell: index in the field, and along x
@@ -249,7 +257,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_list_sp(const __grid_constant
 #pragma unroll
                     for (int e = 0; e < VW; ++e) {
                         any |= !is_exact_zero(cv[q][e]);
-                        inter |= (above_zero(cv[q][e]) && !at_least_one(cv[q][e]) ? 1u : 0u) << e;
+                        inter |= (holds<VW>(cv[q][e]) && !at_least_one(cv[q][e]) ? 1u : 0u) << e;
                         occ |= (above(cv[q][e], tau) ? 1u : 0u) << e;
                     }
                     const unsigned vote = __ballot_sync(0xffffffffu, valid && any);
@@ -434,7 +442,7 @@ __global__ void __launch_bounds__(kSweepThreads, 4)
             for (int e = 0; e < VW; ++e) {
                 const int sl = vsign(ulo[e]), sh = vsign(uhi[e]);
                 const T dl = sl > 0 ? cl[e] : cx[e], dh = sh < 0 ? ch[e] : cx[e];
-                const bool ml = valid && sl != 0 && above_zero(dl), mh = valid && sh != 0 && above_zero(dh);
+                const bool ml = valid && sl != 0 && holds<VW>(dl), mh = valid && sh != 0 && holds<VW>(dh);
                 full_lo[e] = ml && at_least_one(dl);
                 full_hi[e] = mh && at_least_one(dh);
                 F_lo[e] = F_hi[e] = T(0);
@@ -472,7 +480,7 @@ __global__ void __launch_bounds__(kSweepThreads, 4)
                     occm |= (valid && above(v[e], tau) ? 1u : 0u) << e;
                 }
                 nonzero |= !is_exact_zero(v[e]);
-                if (above_zero(v[e]) && !at_least_one(v[e])) {
+                if (holds<VW>(v[e]) && !at_least_one(v[e])) {
                     flo |= (valid && vsign(unl[e]) < 0 ? 1u : 0u) << e;
                     fhi |= (valid && vsign(unh[e]) > 0 ? 1u : 0u) << e;
                 }
