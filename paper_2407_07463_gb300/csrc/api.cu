@@ -42,7 +42,7 @@ enum Slot {
     S_CEN,
     S_VOL,
     S_ROOT,
-    S_HIST_R,
+    S_HIST_R,  // the three accumulators, cleared together
     S_HIST_RT,
     S_MOM,
     S_SHAPE,
@@ -606,9 +606,9 @@ vof_status vof_init(const vof_config* cfg, void* c_dev, const void* u_dev, void*
     if (cudaMemsetAsync(ctx->ws + L.off[S_MISC], 0, kMiscBytes, ctx->stream) != cudaSuccess ||
         (ctx->fp64 ? clear_set_fp64(ctx_box_set<double>(ctx, nullptr, 0.0), ctx->stream)
                    : clear_set_fp32(ctx_box_set<float>(ctx, nullptr, 0.0), ctx->stream)) != cudaSuccess ||
-        cudaMemsetAsync(ctx->ws + L.off[S_HIST_R], 0, L.size[S_HIST_R], ctx->stream) != cudaSuccess ||
-        cudaMemsetAsync(ctx->ws + L.off[S_HIST_RT], 0, L.size[S_HIST_RT], ctx->stream) != cudaSuccess ||
-        cudaMemsetAsync(ctx->ws + L.off[S_MOM], 0, L.size[S_MOM], ctx->stream) != cudaSuccess) {
+        // the histograms and the moments lie side by side
+        cudaMemsetAsync(ctx->ws + L.off[S_HIST_R], 0, L.off[S_MOM] + L.size[S_MOM] - L.off[S_HIST_R], ctx->stream) !=
+            cudaSuccess) {
         (void)cudaGetLastError();
         delete ctx;
         return VOF_ERR_CUDA;
