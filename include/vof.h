@@ -481,7 +481,12 @@ vof_status vof_batch_set_mlp(vof_batch *batch, const void *weights_dev, double f
 /* Times the update launch shapes on the batch's next sweep (the state is
  * not modified) and keeps the fastest; the next step lists its faces afresh. */
 vof_status vof_batch_tune(vof_batch *batch);
-/* nsteps steps of every box, asynchronous on the batch's stream. */
+/* nsteps steps of every box, asynchronous on the batch's stream.  Between
+ * calls the boxes' c must not be changed: the list of interfacial faces and the
+ * map of non-zero words are kept from step to step, and cells put into empty
+ * words are not advanced (a context lists afresh in every vof_step).  After a
+ * change, make the batch anew or call vof_batch_tune, after which the next step
+ * lists afresh.  The velocities are scanned by vof_batch_init only. */
 vof_status vof_batch_step(vof_batch *batch, int32_t nsteps);
 /* Synchronises; VOF_ERR_TIMEOUT if a tensor-core wait gave up. */
 vof_status vof_batch_report(vof_batch *batch, vof_batch_report_t *report);

@@ -555,7 +555,8 @@ class Batch:
     """Independent boxes advanced together (one launch per sweep pass for
     every box, graph replay, tuned update launch shape).  boxes: list of
     (c, u, dt) with c [K][nz][ny][nx] and u [3][nz][ny][nx] device tensors
-    of the precision's dtype; k_active: list or None (all fields)."""
+    of the precision's dtype; k_active: list or None (all fields).  c must not
+    be changed between steps (make a new batch, or call tune())."""
 
     def __init__(self, boxes, precision=VOF_MIXED, k_active=None, h=1.0, tag_tau=1e-6, band=1e-3,
                  use_graph=True, autotune=True, stream=None):
