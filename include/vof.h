@@ -260,7 +260,6 @@ vof_status vof_curvature(vof_ctx *ctx, int32_t field, void *kappa_dev);
 vof_status vof_surface_tension(vof_ctx *ctx, double gamma, void *f_dev);
 
 /*
- * Drop shape (Appendix A)/*
  * Drop shape (Appendix A): the inertia tensor of each drop about its centre
  * of mass, I = integral over the drop of [(r.r) delta - r r], r = x - x_cen
  * under the minimum image, for the drop's colour density (each cell of the

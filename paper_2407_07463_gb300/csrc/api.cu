@@ -494,7 +494,6 @@ vof_status stats_accumulate(vof_ctx* ctx, long long* D_out, double* vtot_out) {
     const Dims& g = ctx->g;
     const vof_config& cf = ctx->cfg;
     cudaStream_t st = ctx->stream;
-    size_t words = (size_t)g.rows * g.W;
     double* hr = ctx->slot<double>(S_HIST_R);
     double* hrt = ctx->slot<double>(S_HIST_RT);
     double* mom = ctx->slot<double>(S_MOM);
@@ -1078,7 +1077,7 @@ const char* vof_last_cuda_error(void) { return vof::last_cuda_error_name(); }
 const char* vof_profile_class_name(int32_t cls) {
     static const char* names[P_COUNT] = {"list_faces", "face_flux", "update", "pack_bits", "near_contact",
                                          "label",      "pairs",     "touch",  "move",      "stats",
-                                         "misc",       "net_normals", "scan"};
+                                         "misc",       "net_normals"};
     if (cls < 0 || cls >= P_COUNT) return nullptr;
     return names[cls];
 }

@@ -2,10 +2,10 @@
 // up to kMaxBoxes for a batch): every pass of a sweep is one launch that
 // covers every field of every box.
 //
-// The set travels by value as a __grid_constant__ kernel parameter (about
-// 8 KB for 64 boxes; read in place from the parameter space), so a
-// captured CUDA graph holds it and no table has to be copied to the
-// device.
+// The set travels by value as a __grid_constant__ kernel parameter (10.8 KB
+// for 64 boxes in FP32, 11.3 KB in double; read in place from the parameter
+// space), so a captured CUDA graph holds it and no table has to be copied to
+// the device.
 //
 // The sweep passes work on words: 32 consecutive cells of a row of one field
 // (the unit of the occupancy bits), VW cells per lane and 32 / VW lanes per
@@ -86,6 +86,8 @@ struct BoxSet {
     BoxDev<T> b[NB];
 };
 
+static_assert(sizeof(BoxSet<double, kMaxBoxes>) <= 16 * 1024, "well within the 32 KB of kernel parameters");
+
 template <typename T, int NB>
 __device__ __forceinline__ int box_of_tile(const BoxSet<T, NB>& S, int tile) {
     if (NB == 1) return 0;
@@ -117,12 +119,12 @@ __device__ __forceinline__ uint16_t* nz_out(const BoxDev<T>& B, int sweep) {
 }
 
 // Words of a tile: most, and the number for a set of `words` words in all --
-// smaller tiles until they outnumber the blocks a GPU holds several times.
+// smaller tiles until there are eight to an SM, twice what it holds at once.
 constexpr int kTileWords = 128;
 constexpr int kSweepThreads = 256;
 inline int tile_words(long long words) {
     int tw = kTileWords;
-    while (tw > 16 && words / tw < 1216) tw /= 2;
+    while (tw > 16 && words / tw < 8 * sm_count()) tw /= 2;
     return tw;
 }
 

@@ -171,9 +171,7 @@ __global__ void __launch_bounds__(kJudgeTile, 8) k_face_flux_judged(const __grid
         const unsigned qb = __ballot_sync(0xffffffffu, queue);
         if (lane == 0) s_wq[warp] = __popc(qb);
         __syncthreads();
-        int q_off = 0;
-#pragma unroll
-        int nq = 0;
+        int q_off = 0, nq = 0;
 #pragma unroll
         for (int w = 0; w < kJudgeWarps; ++w) {
             q_off += w < warp ? s_wq[w] : 0;
@@ -226,9 +224,7 @@ __global__ void __launch_bounds__(kJudgeTile, 8) k_face_flux_judged(const __grid
             s_m[2][t] = m[2];
         }
         __syncthreads();
-        int b_off = 0;
-#pragma unroll
-        int nb = 0;
+        int b_off = 0, nb = 0;
 #pragma unroll
         for (int w = 0; w < kJudgeWarps; ++w) {
             b_off += w < warp ? s_wq[w] : 0;

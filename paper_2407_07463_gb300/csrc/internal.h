@@ -24,7 +24,6 @@ enum ProfClass {
     P_STATS,
     P_MISC,
     P_NET_NORMALS,
-    P_SCAN,
     P_COUNT
 };
 

@@ -107,13 +107,13 @@ __device__ __forceinline__ float dvol_pw(const VolPW& p, float alpha) {
     return alpha <= 0.f || alpha >= p.S ? 0.f : d;
 }
 
-// Root in (0, S/2] of vol_pw = v, 0 < v <= 1/2: the regions of alpha_sorted
-// below, each in closed form -- regions 1 and 2 by a cube and a square
-// root, the prism linearly, and the cubics of regions 3 (b < alpha <=
+// Root in (0, S/2] of vol_pw = v, 0 < v <= 1/2, region by region in closed
+// form: 1 (alpha <= a) and 2 (a < alpha <= b) by a cube and a square root, 5
+// (the prism, a + b < alpha <= c) linearly, the cubics of 3 (b < alpha <=
 // min(c, a + b)) and 4 (c < alpha <= S/2) by their middle real root
-// (trigonometric form), which one Newton step on vol_pw then polishes.
-// Products by the normal's constants replace divisions.  *region as for
-// alpha_sorted.
+// (trigonometric form); one Newton step on vol_pw then polishes the root.
+// Products by the normal's constants replace divisions.  *region (if not
+// null) receives the number, 0 for a plane parallel to an axis.
 //
 // Region 3: alpha^3 - (alpha-a)^3 - (alpha-b)^3 = 6abc v becomes, with
 // alpha = a + b + t, t^3 - 6ab t + 3ab (2cv - a - b) = 0.  Region 4 (the c
@@ -121,9 +121,9 @@ __device__ __forceinline__ float dvol_pw(const VolPW& p, float alpha) {
 // 3abc (v - 1/2) = 0, e2 = ab + bc + ca.  Both have three real roots, t =
 // 2r cos(acos(z)/3 - 2 pi k/3) with r^2 = -p/3 and z = -q / (2 r^3); the
 // root of the region is the middle one (k = 1).  Measured against Newton
-// from the region's end (the earlier form): the same error against the FP64
-// inversion (1.4e-7) and 18% fewer issue slots, the Newton loop's trip
-// count diverging within a warp.
+// from the region's end: the same error against the FP64 inversion (1.4e-7)
+// and 18% fewer issue slots, the Newton loop's trip count diverging within a
+// warp.
 static __device__ __noinline__ float alpha_sorted_pw(const VolPW p, float v, int* region = nullptr) {
     const float a = p.a, b = p.b, c = p.c;
     if (a <= kTinyF) {

@@ -305,7 +305,7 @@ __device__ __forceinline__ double image_shift(double t, double L) {
 }
 
 // A run of `cnt` cells from (i, j, k) (cell x) whose drop is `idx`: its share
-// added to the drop by itself (runs that a strip's sums do not take).
+// added to the drop.
 template <typename T, DropMode MODE>
 __device__ __forceinline__ void add_run(const T* __restrict__ cf, const Dims& g, const DropOut& o, int idx, int x, int i,
                                         int j, int k, int cnt, const RunSums<T>& rs) {
@@ -433,18 +433,16 @@ __global__ void __launch_bounds__(32 * kDropWarps) k_drop_words(const __grid_con
         __syncwarp();
         for (int base = 0; base < n; base += 32) {
             const int have = min(32, n - base);
-            if (MODE != DropRoots || !BITS) {
 #pragma unroll 8
-                for (int q = 0; q < have; ++q) {
-                    int x0, cells;
-                    place(s_word[wp][base + q], x0, cells);
-                    if (lane < cells) {
-                        if (MODE != DropRoots) s_c[wp][lane][q] = cf[x0 + lane];
-                        if (!BITS) s_lab[wp][lane][q] = lab[x0 + lane];
-                    }
+            for (int q = 0; q < have; ++q) {
+                int x0, cells;
+                place(s_word[wp][base + q], x0, cells);
+                if (lane < cells) {
+                    if (MODE != DropRoots) s_c[wp][lane][q] = cf[x0 + lane];
+                    if (!BITS) s_lab[wp][lane][q] = lab[x0 + lane];
                 }
-                __syncwarp();
             }
+            __syncwarp();
             if (lane < have) {
                 const int w = s_word[wp][base + lane];
                 uint32_t rest = s_mask[wp][base + lane];
@@ -478,8 +476,13 @@ static void launch_drop_words(const DropFields& D, const Dims& g, const DropOut&
     while (rounds > 1 && words * D.ls.n / (32 * rounds) < (long long)sm_count() * 16) rounds /= 2;
     const dim3 grid(grid_for(words, 32 * kDropWarps * rounds, std::max(1, sm_count() * 24 / D.ls.n)), D.ls.n);
     auto go = [&](auto kernel) { kernel<<<grid, 32 * kDropWarps, 0, st>>>(D, g, o, rounds); };
-    if (D.fp64) D.bits ? go(k_drop_words<double, MODE, true>) : go(k_drop_words<double, MODE, false>);
-    else D.bits ? go(k_drop_words<float, MODE, true>) : go(k_drop_words<float, MODE, false>);
+    if constexpr (MODE != DropRoots) {  // (the roots come from labels alone)
+        if (D.bits) {
+            D.fp64 ? go(k_drop_words<double, MODE, true>) : go(k_drop_words<float, MODE, true>);
+            return;
+        }
+    }
+    D.fp64 ? go(k_drop_words<double, MODE, false>) : go(k_drop_words<float, MODE, false>);
 }
 
 cudaError_t drop_roots(const DropFields& D, const Dims& g, int* root_of, cudaStream_t st) {
