@@ -164,11 +164,11 @@ def peaks():
 
 
 def algorithmic_bytes(cls, n_cells, fields, es):
-    """Minimum DRAM bytes one launch of a kernel class must move.
+    """DRAM bytes of one launch of a kernel class that touches every cell once.
     update (one sweep of every active field): read c_in and write c_out per
     cell-field, one c_c bit read or written and (last sweep) one occupancy
     bit per cell-field, the sweep's and the next sweep's velocity component
-    per cell.  list_faces: read c per cell-field plus one velocity
+    per cell; the pass skips words that cannot change and moves less.  list_faces: read c per cell-field plus one velocity
     component.  pack_bits: read c per cell-field, write one bit.
     near_contact: read and write one bit per cell-field."""
     if cls == "update":
@@ -662,10 +662,12 @@ def run_ours(args, rank, world):
             roof = r
         if name == "update":
             own = algorithmic_bytes("update", N, fields, es)
-            roof_update = dict(r, algorithmic_bytes_per_launch=own, achieved=own / (tot / cnt * 1e-3) / 1e9,
-                               basis="bytes of a pass over every word (c in and out, bits, velocities); "
-                                     "words that cannot change are skipped: an equivalent rate, not traffic")
-            roof_update["frac"] = roof_update["achieved"] / hbm
+            roof_update = {"kernel": name, "bound": "latency", "launches": cnt, "avg_ms": tot / cnt,
+                           "share_of_timed": tot / ms, "traffic": traffic_tab.get(name),
+                           "dense_bytes_per_launch": own,
+                           "equivalent_rate": own / (tot / cnt * 1e-3) / 1e9, "unit": "GB/s",
+                           "basis": "bytes of a pass over every word (c in and out, bits, velocities) over the time; "
+                                    "words that cannot change are skipped: neither traffic nor a share of a peak"}
         if name == "face_flux" and prec == vof.VOF_MIXED_LEARNED:
             roof_alu = alu_roofline(cnt, tot, rep, sm_count, sm_mhz)
         if name == "net_normals":
