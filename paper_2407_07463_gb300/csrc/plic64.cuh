@@ -259,11 +259,43 @@ VOF_HD double scaled64(long long n, int sh) {
     return from_bits64(n < 0 ? b | (long long)0x8000000000000000ULL : b);
 }
 
-// The rule evaluated in double, for the stencils below.
+// The rule evaluated in double, for the stencils below: as it stands, and for
+// values of fractions' size (a few divisions instead of seven: quotients are
+// formed only where rounding may decide, and a common factor is left in).
 VOF_HD_CALL void myc_rule64(const double* st, double m[3]) { myc_normal<double>(st, m); }
+VOF_HD_CALL void myc_tie64(const double* st, double m[3]) {
+    double y[3];
+    youngs_raw(st, y);
+    centred_column(st, 0, y, m);
+    double l = l1norm(m);
+VOF_UNROLL
+    for (int a = 1; a < 3; ++a) {
+        double r[3];
+        centred_column(st, a, y, r);
+        const double n = l1norm(r);
+        // 1 / n > 1 / l, which differ if n and l do by two ulps
+        if (n < l && (l - n > 5e-16 * l || 1.0 / n > 1.0 / l)) {
+            l = n;
+            m[0] = r[0];
+            m[1] = r[1];
+            m[2] = r[2];
+        }
+    }
+    const double ny = l1norm(y);
+    if (!(ny >= 1e-30)) return;
+    const double y01 = lt_pos(abs64(y[0]), abs64(y[1])) ? abs64(y[1]) : abs64(y[0]);
+    const double ymax = lt_pos(y01, abs64(y[2])) ? abs64(y[2]) : y01;
+    const double gap = ny - ymax * l;  // ymax / ny < 1 / l
+    if (abs64(gap) > 1e-14 * ny ? gap > 0.0 : ymax / ny < 1.0 / l) {
+        const double il = 1.0 / ny;
+        m[0] = y[0] * il;
+        m[1] = y[1] * il;
+        m[2] = y[2] * il;
+    }
+}
 
 // Mixed-Youngs-Centred direction of a stencil (myc.cuh gives the rule), not
-// normalised: its largest component lies in 1/3 .. 2.  The hundred additions run
+// normalised: its largest component lies in 1/3 .. 96.  The hundred additions run
 // on 64-bit integers (the integer pipes are idle in the FP64 kernels): the
 // fractions become whole numbers of 2^-57 of the largest neighbour's binade, 32
 // times finer than that value's own last place, so that sums and differences are
@@ -382,7 +414,7 @@ VOF_HD void myc_direction64(const double* st, double m[3], double edge) {
     const unsigned long long own_y = axis == 0 ? ax : (axis == 1 ? ay : az);
     open = open || ymax < (1ull << 36) || (!youngs && own_y < (1ull << 15));
     if (open && any != 0 && le_pos(edge, plus64(st[13])) && le_pos(edge, plus64(1.0 - st[13]))) {
-        myc_rule64(st, m);
+        myc_tie64(st, m);
         return;
     }
     // Youngs' largest component goes to 1 .. 2
