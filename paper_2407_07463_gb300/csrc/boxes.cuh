@@ -648,9 +648,10 @@ __global__ void __launch_bounds__(256) k_list_patch(const __grid_constant__ BoxS
 // reordered so that a warp runs one piece, at most two, instead of all three
 // with nine lanes each), took it from 6.2 to 0.72 ms per sweep of the 256^3,
 // K = 8, phi = 0.3 box (2.7 M faces; 1.08 ms before the reordering and before
-// the volume's pieces became selects: 212 -> 88 to 120 FP64 instructions per
-// warp of faces), and a sweep of 32^3 with 8 drops, where one warp's chain is
-// the time, from 78 to 20 us with its other launches.
+// the volume's pieces became selects), and a sweep of 32^3 with 8 drops, where
+// one warp's chain is the time, from 78 to 20 us with its other launches.  0.55 ms
+// since the normals near a tie go to a call and fluxes of donors a few ulps from
+// 1 do without (84 FP64 instructions per warp of faces in the first sweep).
 //
 // In FP32 the faces whose fraction lies within `band` of 0 or 1 (one in six)
 // take an FP64 step: they are compacted to the first threads of the block, so

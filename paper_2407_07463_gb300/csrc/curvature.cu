@@ -23,7 +23,7 @@
 // for the curvatures and 0.16 ms for the source (0.18 ms with three fields'
 // values held in flight: fewer warps); a thread per cell took 2.19 ms for the
 // curvatures (few lanes of a warp gathering, an index modulo per value) and
-// 0.40 ms for the source.
+// 0.40 ms for the source.  In double 0.48 and 1.12 ms, bound by FP64 issue.
 #include <algorithm>
 #include <type_traits>
 
